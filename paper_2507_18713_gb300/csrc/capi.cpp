@@ -44,11 +44,37 @@ extern "C" salf_status salf_create(int32_t device, salf_ctx** out) {
   if (st != SALF_OK) return st;
   salf_ctx* c = new salf_ctx();
   c->device = device;
+  cudaMemPoolProps props;
+  std::memset(&props, 0, sizeof(props));
+  props.allocType = cudaMemAllocationTypePinned;
+  props.handleTypes = cudaMemHandleTypeNone;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = device;
+  unsigned long long keep = kPoolKeep;
+  if ((e = cudaMemPoolCreate(&c->pool, &props)) != cudaSuccess ||
+      (e = cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+    salf_destroy(c);
+    return salf_cuda_fail(e, "cudaMemPoolCreate");
+  }
   *out = c;
   return SALF_OK;
 }
 
-extern "C" void salf_destroy(salf_ctx* ctx) { delete ctx; }
+extern "C" void salf_destroy(salf_ctx* ctx) {
+  if (!ctx) return;
+  if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
+  delete ctx;
+}
+
+salf_status PoolBuf::get(salf_ctx* ctx, size_t bytes, cudaStream_t stream) {
+  const cudaError_t e = cudaMallocFromPoolAsync(&p, bytes ? bytes : 16, ctx->pool, stream);
+  if (e != cudaSuccess) {
+    p = nullptr;
+    return salf_cuda_fail(e, "cudaMallocFromPoolAsync");
+  }
+  st = stream;
+  return SALF_OK;
+}
 
 extern "C" salf_status salf_build_scene(salf_ctx* ctx, const salf_scene_desc* desc,
                                         salf_scene** out) {
@@ -68,7 +94,7 @@ extern "C" void salf_scene_destroy(salf_scene* s) {
   if (!s) return;
   cudaSetDevice(s->device);
   cudaDeviceSynchronize();
-  for (void* p : s->allocations) cudaFree(p);
+  for (void* p : s->allocations) cudaFreeAsync(p, 0);  // the device is idle
   if (s->staging) cudaFree(s->staging);
   if (s->grads) cudaFree(s->grads);
   if (s->raster_vox) cudaFree(s->raster_vox);
@@ -146,7 +172,6 @@ extern "C" salf_status salf_scene_check(salf_scene* s) {
   if (flag) {
     cudaMemset(s->dev.status, 0, sizeof(int));
     g_err = "device status word " + std::to_string(flag) +
-            ((flag & SALF_DEVERR_STEP_CAP) ? " (traversal step bound reached)" : "") +
             ((flag & SALF_DEVERR_SDF_AB) ? " (SDF record with a <= 0 or b <= 0)" : "") +
             ((flag & SALF_DEVERR_ACTOR_CAP) ? " (a ray met more actor boxes than it holds)" : "") +
             ((flag & SALF_DEVERR_BOUNDS) ? " (an adjoint index outside its buffers, skipped)" : "");

@@ -62,8 +62,10 @@ salf_status salf_scene_keep_keys(salf_scene* s, const salf_scene_desc* d) {
   st = salf_scene_dalloc(s, (size_t)n * 3 * sizeof(int32_t), &ij);
   if (st != SALF_OK) return st;
   const cudaMemcpyKind k = d->keys_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-  cudaError_t e = cudaMemcpy(lv, d->level, (size_t)n, k);
-  if (e == cudaSuccess) e = cudaMemcpy(ij, d->ijk, (size_t)n * 3 * sizeof(int32_t), k);
+  cudaError_t e = cudaMemcpyAsync(lv, d->level, (size_t)n, k, 0);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(ij, d->ijk, (size_t)n * 3 * sizeof(int32_t), k, 0);
+  // the caller may free its arrays, and use the scene on any stream, from here on
+  if (e == cudaSuccess) e = cudaStreamSynchronize(0);
   if (e != cudaSuccess) return salf_cuda_fail(e, "scene keys copy");
   s->key_level = static_cast<const uint8_t*>(lv);
   s->key_ijk = static_cast<const int32_t*>(ij);

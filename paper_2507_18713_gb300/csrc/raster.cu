@@ -234,19 +234,20 @@ __global__ void __launch_bounds__(kRasterThreads, SALF_RASTER_MIN_BLOCKS) k_rast
   const int ray = v * Q.W + u;
 
   Ray r;
-  Walk w;
-  w.alive = false;
+  RayClip w;
+  bool alive = false;
   r.valid = false;
   r.d[0] = r.d[1] = r.d[2] = 0.f;
   if (in_img) {
     gen_ray_pinhole(Q, u, v, r);  // the rasteriser serves pinhole cameras with one pose
-    walk_init(S, r, w);
+    ray_clip(S, r, w);
+    alive = r.valid && w.t0 < w.t1;
   }
   float gam[4];
   sh_basis(r.d, gam);
   const bool want_int = Q.want_int != 0;
   const float tmin = Q.t_min;
-  const float t0 = w.t;
+  const float t0 = w.t0;
   bool pos[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) pos[a] = w.D[a] > 0.f;
@@ -301,14 +302,14 @@ __global__ void __launch_bounds__(kRasterThreads, SALF_RASTER_MIN_BLOCKS) k_rast
       // the exit is the nearest exit plane (the ray kernel's tx[ax]: the same value, as the
       // distances are finite), taken as a minimum so the distances stay in registers
       *tin_out = tin;
-      *tout_out = fminf(fminf(fminf(tx[0], tx[1]), tx[2]), w.tend);
+      *tout_out = fminf(fminf(fminf(tx[0], tx[1]), tx[2]), w.t1);
     };
     // phase 1: which of the strip's voxels this pixel's ray crosses
     unsigned hits[kChunk / 32];
 #pragma unroll
     for (int q = 0; q < kChunk / 32; ++q) {
       hits[q] = 0u;
-      unsigned m = w.alive ? sel[q] : 0u;
+      unsigned m = alive ? sel[q] : 0u;
       while (m) {
         const int jj = __ffs(m) - 1;
         m &= m - 1;
@@ -323,32 +324,33 @@ __global__ void __launch_bounds__(kRasterThreads, SALF_RASTER_MIN_BLOCKS) k_rast
     // phase 2: the lanes composite their next hit together, in list order
 #pragma unroll
     for (int q = 0; q < kChunk / 32; ++q) {
-      while (__any_sync(0xffffffffu, w.alive && hits[q] != 0u)) {
-        if (w.alive && hits[q]) {
+      while (__any_sync(0xffffffffu, alive && hits[q] != 0u)) {
+        if (alive && hits[q]) {
           const int jj = __ffs(hits[q]) - 1;
           hits[q] &= hits[q] - 1;
           const int j = q * 32 + jj;
           float tin, tout;
           slab(j, &tin, &tout);
           const int4 b = s_box[j];
-          Hit h;
-          h.vox = s_vox[j];
-          h.ls = b.w;
-          h.base[0] = b.x;
-          h.base[1] = b.y;
-          h.base[2] = b.z;
-          h.tin = tin;
-          h.tout = tout;
-          composite_hit<DT, MODE>(w, h, SharedRec{&s_rec[j * RS]}, want_int, gam, A);
+          // local coordinates of the midpoint, as the ray kernel forms them
+          const float tm = 0.5f * (tin + tout);
+          const float E = (float)(1 << b.w);
+          const float inv_half = __int_as_float((128 - b.w) << 23);  // 2 / E
+          const int lo[3] = {b.x, b.y, b.z};
+          float x[3];
+#pragma unroll
+          for (int a = 0; a < 3; ++a)
+            x[a] = (fmaf(tm, w.D[a], Q.Of[a]) - ((float)(lo[a] - Q.Oi[a]) + 0.5f * E)) * inv_half;
+          composite_at<DT, MODE>(x, tm, tout - tin, SharedRec{&s_rec[j * RS]}, want_int, gam, A);
           if (DUMP) {
-            if (A.nvis < Q.vcap) Q.visits[(size_t)ray * Q.vcap + A.nvis] = __ldg(&S.order[h.vox]);
+            if (A.nvis < Q.vcap) Q.visits[(size_t)ray * Q.vcap + A.nvis] = __ldg(&S.order[s_vox[j]]);
           }
           ++A.nvis;
-          if (A.T < tmin) w.alive = false;
+          if (A.T < tmin) alive = false;
         }
       }
     }
-    if (__syncthreads_count(w.alive) == 0) break;
+    if (__syncthreads_count(alive) == 0) break;
   }
   if (!in_img) return;
   write_outputs(Q, ray, r.valid, A);

@@ -163,8 +163,8 @@ __global__ void __launch_bounds__(256) k_reg_loss(const __grid_constant__ DevSce
       int c[3] = {lo[0], lo[1], lo[2]};
       c[ax] = sgn > 0 ? lo[ax] + E : lo[ax] - 1;
       if (c[ax] < 0 || c[ax] >= S.Gf[ax]) continue;
-      int lsj;
-      const int j = salf::find_leaf(S, c[0], c[1], c[2], &lsj);
+      int lsj, lz;
+      const int j = salf::find_leaf(S, c[0], c[1], c[2], &lsj, &lz);
       if (j < 0 || lsj < bi.w || (lsj == bi.w && sgn < 0)) continue;
       const int4 bj = __ldg(&S.vox_box[j]);
       const int Ej = 1 << bj.w;

@@ -127,10 +127,13 @@ __global__ void __launch_bounds__(32 * WPB, MINB) k_forward(const __grid_constan
   float T_prev = 1.f;  // SEG: this span's T before its last composited hit
   bool keep = true;    // SEG: the whole ray reaches this lane's span
 
+  int steps = 0;       // DUMP: structure steps of the ray
+
   for (int pass = 0;; ++pass) {
     for (;;) {
       Hit h;
-      bool hit = next_hit<!SEG>(S, w, h);
+      if (DUMP) steps += w.alive ? 1 : 0;
+      bool hit = next_hit(S, w, h);
       if (SEG && !hit && w.t > walk_end) w.alive = false;  // the rest is the next span's
       if (!__any_sync(0xffffffffu, hit || w.alive)) break;
       if (SEG && hit && ks > 0) {  // composite only the voxels entered inside this span
@@ -209,7 +212,7 @@ __global__ void __launch_bounds__(32 * WPB, MINB) k_forward(const __grid_constan
   if (!in_img) return;
   write_outputs(Q, ray, r.valid, A, want_drop);
   if (DUMP) {
-    if (Q.steps_out) Q.steps_out[ray] = w.steps;
+    if (Q.steps_out) Q.steps_out[ray] = steps;
     if (Q.vcap > 0) {
       Q.vcount[ray] = A.nvis;
       for (int k = A.nvis; k < Q.vcap; ++k) Q.visits[(size_t)ray * Q.vcap + k] = -1;

@@ -11,8 +11,6 @@
 
 #include "../../include/salf.h"
 
-#define SALF_MAX_MASK_LEVELS 12
-#define SALF_MAX_COL_LEVELS 16
 #define SALF_MAX_BATCH 24
 #ifndef SALF_TILE_W
 #define SALF_TILE_W 8  // camera warp tile: SALF_TILE_W x (32 / SALF_TILE_W) pixels
@@ -36,7 +34,6 @@
 #endif
 
 // Device status-word bits.
-#define SALF_DEVERR_STEP_CAP 1  // a traversal loop reached its iteration bound
 #define SALF_DEVERR_SDF_AB 2    // an SDF record has a <= 0 or b <= 0
 #define SALF_DEVERR_ACTOR_CAP 4 // a ray met more actor boxes than it can hold
 #define SALF_DEVERR_BOUNDS 8    // an adjoint kernel met an index outside its buffers (skipped)
@@ -44,40 +41,38 @@
 // Read-only view of a built scene, passed to kernels by value.
 //
 // Acceleration structure (replaces the paper's pointer octree, Sec. III-B):
-//  * occupancy pyramid: mask level 0 has one 64-bit word per 4x4x4 block of
-//    level-0 cells (bit = Morton index of the cell inside the block) plus the
-//    rank offset of the block's first occupied cell in `cells` and, when
-//    every occupied cell of the block is one level-0 voxel, the index of the
-//    block's first voxel (voxels are numbered block by block, cells inside a
-//    block in bit order), else all ones; mask level
-//    m >= 1 has one word per 4x4x4 words of level m-1 (bit set iff that word
-//    is non-zero).  An empty cell is skipped together with the largest empty
-//    aligned pyramid cell that contains it (one slab exit per skip).
+//  * occupancy: one 64-bit word per 4x4x4 block of level-0 cells (bit = Morton
+//    index of the cell inside the block) plus the rank offset of the block's
+//    first occupied cell in `cells` and, when every occupied cell of the block
+//    is one level-0 voxel, the index of the block's first voxel (voxels are
+//    numbered block by block, cells inside a block in bit order), else all ones.
+//  * skip boxes: the voxels' tight box is cut into bricks of 4x4x1 level-0
+//    cells (larger ones in very large grids).  For each of the 8 direction
+//    octants, an empty brick holds the size of an empty box that starts at it
+//    and extends in the octant's directions (ex | ey << 5 | ez << 10 bricks,
+//    1..31, 1..31, 1..63); a brick with voxels holds 0.  A ray leaves empty
+//    space in one step per box, from one 2-byte read.
 //  * cells[rank] = (e, cm) for each occupied level-0 cell.  cm == 0: e is a
 //    voxel index (>= 0) or -2 - node for a subdivided cell; nodes hold 8
 //    children with the same encoding (-1 = empty child).  cm != 0: the cell is
 //    split once into voxels; cm is the occupancy of its 8 children (bit =
 //    x | y << 1 | z << 2) and child c is voxel e + popcount(cm & ((1 << c) - 1)).
-//  * column pyramid: for every footprint of 2^c x 2^c level-0 columns, a
-//    128-bit mask of the z-layers (layer = layer_cells level-0 cells high)
-//    that hold any voxel.  A ray in an empty layer of a footprint can jump to
-//    the nearest occupied layer in its direction of travel, or to the
-//    footprint's side, in one step.
 //  * params: records in voxel order (block, cell inside the block, Morton
 //    index of the min corner inside the cell), FP32 or BF16;
 //    order[internal] = input index; vox_box[internal] = (min corner in finest
 //    cells, log2 of the edge in finest cells), read by the rasteriser.
 struct DevScene {
   const uint4* mask0;
-  const unsigned long long* mask[SALF_MAX_MASK_LEVELS];
-  int mdim[SALF_MAX_MASK_LEVELS][3];
+  int mdim0, mdim01;  // blocks per row (x) and per layer (x, y)
   const int2* cells;
   const int* nodes;
-  const uint4* col[SALF_MAX_COL_LEVELS];  // column masks per level: (lo64, hi64) as uint4
-  int cdim[SALF_MAX_COL_LEVELS][2];
-  int CL;           // column levels
-  int layer_shift;  // log2(layer height in finest cells)
-  int n_layers;     // <= 128
+  // octant o (bit a: the ray travels downwards on axis a) starts at
+  // o * skip_n01 * skip_n[2], bricks in mirrored order on its downward axes
+  const unsigned short* skip;
+  int skip_n[3], skip_n01;  // bricks per axis; per layer
+  int skip_base[3];         // first brick per axis (brick = cell >> shift)
+  int skip_sx, skip_sz;     // log2 of a brick's edges (x and y; z), finest cells
+  int skip_coarse;          // bricks are larger than a layer of a block
   const void* params;
   const int* order;
   const int4* vox_box;
@@ -85,7 +80,6 @@ struct DevScene {
   double origin[3];
   double inv_sfin;  // finest cells per metre
   int K;
-  int M;
   int Gf[3];
   int bmin[3], bmax[3];  // tight box of all voxels, finest cells [bmin, bmax)
   int mode, dtype;
@@ -176,8 +170,16 @@ struct LaunchParams {
 
 // ---------------------------------------------------------------- host side
 
+// Device memory of scenes and of their builds comes from a pool of the
+// context's own, which keeps up to kPoolKeep freed bytes for the next build
+// (cudaMalloc and cudaFree took more than half of a 1M-voxel rebuild).  The
+// pool goes with the context; memory that is still out then is given back as
+// its scenes are destroyed.
+constexpr unsigned long long kPoolKeep = 1ull << 30;
+
 struct salf_ctx {
   int device;
+  cudaMemPool_t pool = nullptr;
 };
 
 struct salf_scene {
@@ -227,6 +229,19 @@ struct salf_scene {
   const int32_t* key_ijk = nullptr;
 };
 
+// Temporary device memory of one call, ordered on its stream.
+struct PoolBuf {
+  void* p = nullptr;
+  cudaStream_t st = nullptr;
+  PoolBuf() = default;
+  PoolBuf(const PoolBuf&) = delete;
+  PoolBuf& operator=(const PoolBuf&) = delete;
+  salf_status get(salf_ctx* ctx, size_t bytes, cudaStream_t stream);
+  ~PoolBuf() {
+    if (p) cudaFreeAsync(p, st);
+  }
+};
+
 // NVTX ranges around the library's calls (host side: the range holds the
 // call's launches, so profilers attribute its kernels to it).  Header-only
 // NVTX3; a range costs a few nanoseconds when no tool is attached.
@@ -256,6 +271,12 @@ salf_status salf_noalloc_setup(int device);
 salf_status salf_build_scene_impl(salf_ctx* ctx, const salf_scene_desc* d, salf_scene** out);
 // The same build from device-resident level / ijk / params (validated by the caller).
 salf_status salf_build_scene_gpu(salf_ctx* ctx, const salf_scene_desc* d, salf_scene** out);
+// Blocks per axis (mdim) of a grid's occupancy words, and log2 of its skip
+// bricks' edges in level-0 cells (p: x and y, q: z).
+void salf_grid_shape(const int32_t dims[3], int mdim[3], int* p, int* q);
+// The skip boxes of s->dev from its occupancy words and tight box (D.mask0,
+// D.mdim0, D.mdim01, D.bmin, D.bmax, D.K set); asynchronous on `st`.
+salf_status salf_build_skip(salf_scene* s, int p, int q, cudaStream_t st);
 // A device buffer owned (and freed) by the scene.
 salf_status salf_scene_dalloc(salf_scene* s, size_t bytes, void** p);
 // Keep a copy of the build's voxel keys in the scene (for salf_scene_save).

@@ -1,7 +1,7 @@
 // scene_build.cpp -- salf_build_scene: validates the voxel set, sorts it in
-// block order, builds the occupancy pyramid / level-0 cell table /
+// block order, builds the occupancy words / level-0 cell table /
 // subdivision nodes (the accelerator that stands in for the paper's octree,
-// Sec. III-B) and uploads everything to the device.
+// Sec. III-B), uploads everything and has the device add the skip boxes.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -42,10 +42,10 @@ struct Scope {  // frees a half-built scene on error
 
 salf_status dalloc(salf_scene* s, size_t bytes, void** p) {
   if (bytes == 0) bytes = 16;
-  cudaError_t e = cudaMalloc(p, bytes);
+  cudaError_t e = cudaMallocFromPoolAsync(p, bytes, s->ctx->pool, 0);
   if (e != cudaSuccess) {
     *p = nullptr;
-    salf_set_error(std::string("cudaMalloc(") + std::to_string(bytes) + ") failed: " +
+    salf_set_error(std::string("device allocation (") + std::to_string(bytes) + ") failed: " +
                    cudaGetErrorString(e));
     cudaGetLastError();
     return e == cudaErrorMemoryAllocation ? SALF_ERR_OOM : SALF_ERR_CUDA;
@@ -117,8 +117,8 @@ salf_status salf_build_scene_impl(salf_ctx* ctx, const salf_scene_desc* d, salf_
   // level-0 voxels thus follow the occupancy bits, and a block whose occupied
   // cells are all level-0 voxels maps cell -> voxel by a popcount.  Bits: the
   // block index needs 3 (19 - K) at most, the rest 6 + 3 K, so 63 in all.
-  int mdim[SALF_MAX_MASK_LEVELS][3];
-  for (int a = 0; a < 3; ++a) mdim[0][a] = (d->dims[a] + 3) / 4;
+  int mdim[3], brick_p, brick_q;
+  salf_grid_shape(d->dims, mdim, &brick_p, &brick_q);
   std::vector<uint64_t> code((size_t)n);
   const uint64_t fine = (1ULL << K) - 1ULL;
   for (int64_t v = 0; v < n; ++v) {
@@ -138,7 +138,7 @@ salf_status salf_build_scene_impl(salf_ctx* ctx, const salf_scene_desc* d, salf_
     }
     const uint64_t c0[3] = {f[0] >> K, f[1] >> K, f[2] >> K};
     const uint64_t blk =
-        ((c0[2] >> 2) * (uint64_t)mdim[0][1] + (c0[1] >> 2)) * (uint64_t)mdim[0][0] + (c0[0] >> 2);
+        ((c0[2] >> 2) * (uint64_t)mdim[1] + (c0[1] >> 2)) * (uint64_t)mdim[0] + (c0[0] >> 2);
     code[v] = (blk << (6 + 3 * K)) | ((uint64_t)morton6(c0[0] & 3, c0[1] & 3, c0[2] & 3) << (3 * K)) |
               morton3(f[0] & fine, f[1] & fine, f[2] & fine);
   }
@@ -162,12 +162,12 @@ salf_status salf_build_scene_impl(salf_ctx* ctx, const salf_scene_desc* d, salf_
   }
 
   // ---- occupancy of level-0 cells, rank offsets, cell table, nodes
-  const int64_t nb0 = (int64_t)mdim[0][0] * mdim[0][1] * mdim[0][2];
+  const int64_t nb0 = (int64_t)mdim[0] * mdim[1] * mdim[2];
   std::vector<uint64_t> m0((size_t)nb0, 0);
   std::vector<uint32_t> vfirst((size_t)nb0, 0xffffffffu);
   std::vector<uint8_t> split((size_t)nb0, 0);
   auto block_of = [&](int64_t cx, int64_t cy, int64_t cz) {
-    return ((cz >> 2) * mdim[0][1] + (cy >> 2)) * mdim[0][0] + (cx >> 2);
+    return ((cz >> 2) * mdim[1] + (cy >> 2)) * mdim[0] + (cx >> 2);
   };
   for (int64_t p = 0; p < n; ++p) {
     const int32_t v = order[p];
@@ -249,67 +249,6 @@ salf_status salf_build_scene_impl(salf_ctx* ctx, const salf_scene_desc* d, salf_
     if (flat && cm) cells[r] = make_int2(first, (int)cm);
   }
 
-  // ---- upper pyramid levels
-  std::vector<std::vector<uint64_t>> up(1);
-  int M = 1;
-  {
-    std::vector<uint64_t> prev = m0;
-    while (!(mdim[M - 1][0] == 1 && mdim[M - 1][1] == 1 && mdim[M - 1][2] == 1)) {
-      if (M >= SALF_MAX_MASK_LEVELS) {
-        salf_set_error("salf_build_scene: grid too large for the pyramid");
-        return SALF_ERR_INVALID;
-      }
-      for (int a = 0; a < 3; ++a) mdim[M][a] = (mdim[M - 1][a] + 3) / 4;
-      std::vector<uint64_t> cur((size_t)mdim[M][0] * mdim[M][1] * mdim[M][2], 0);
-      for (int64_t wz = 0; wz < mdim[M - 1][2]; ++wz)
-        for (int64_t wy = 0; wy < mdim[M - 1][1]; ++wy)
-          for (int64_t wx = 0; wx < mdim[M - 1][0]; ++wx) {
-            if (!prev[(wz * mdim[M - 1][1] + wy) * mdim[M - 1][0] + wx]) continue;
-            cur[((wz >> 2) * mdim[M][1] + (wy >> 2)) * mdim[M][0] + (wx >> 2)] |=
-                1ULL << morton6(wx & 3, wy & 3, wz & 3);
-          }
-      up.push_back(cur);
-      prev.swap(cur);
-      ++M;
-    }
-  }
-
-  // ---- column pyramid: z-layer occupancy per footprint of 2^c x 2^c columns
-  int layer_cells = 1;
-  while ((d->dims[2] + layer_cells - 1) / layer_cells > 128) layer_cells *= 2;
-  const int n_layers = (d->dims[2] + layer_cells - 1) / layer_cells;
-  int cdim[SALF_MAX_COL_LEVELS][2];
-  cdim[0][0] = d->dims[0];
-  cdim[0][1] = d->dims[1];
-  std::vector<std::vector<uint4>> cols(1);
-  cols[0].assign((size_t)cdim[0][0] * cdim[0][1], make_uint4(0, 0, 0, 0));
-  for (int64_t p = 0; p < n; ++p) {
-    const int32_t v = order[p];
-    const int l = d->level[v];
-    const int64_t cx = d->ijk[3 * v] >> l, cy = d->ijk[3 * v + 1] >> l, cz = d->ijk[3 * v + 2] >> l;
-    const int layer = (int)(cz / layer_cells);
-    uint4& m = cols[0][(size_t)cy * cdim[0][0] + cx];
-    unsigned* wds = &m.x;
-    wds[layer >> 5] |= 1u << (layer & 31);
-  }
-  int CL = 1;
-  while ((cdim[CL - 1][0] > 1 || cdim[CL - 1][1] > 1) && CL < SALF_MAX_COL_LEVELS) {
-    cdim[CL][0] = (cdim[CL - 1][0] + 1) / 2;
-    cdim[CL][1] = (cdim[CL - 1][1] + 1) / 2;
-    std::vector<uint4> cur((size_t)cdim[CL][0] * cdim[CL][1], make_uint4(0, 0, 0, 0));
-    for (int64_t y = 0; y < cdim[CL - 1][1]; ++y)
-      for (int64_t x = 0; x < cdim[CL - 1][0]; ++x) {
-        const uint4 a = cols[CL - 1][(size_t)y * cdim[CL - 1][0] + x];
-        uint4& b = cur[(size_t)(y >> 1) * cdim[CL][0] + (x >> 1)];
-        b.x |= a.x;
-        b.y |= a.y;
-        b.z |= a.z;
-        b.w |= a.w;
-      }
-    cols.push_back(std::move(cur));
-    ++CL;
-  }
-
   // ---- device upload
   salf_scene* s = new salf_scene();
   Scope guard{s};
@@ -334,13 +273,8 @@ salf_status salf_build_scene_impl(salf_ctx* ctx, const salf_scene_desc* d, salf_
   uint4* dmask0 = nullptr;
   if ((st = upload(s, mask0, &dmask0)) != SALF_OK) return st;
   D.mask0 = dmask0;
-  for (int m = 1; m < M; ++m) {
-    uint64_t* p = nullptr;
-    if ((st = upload(s, up[m], &p)) != SALF_OK) return st;
-    D.mask[m] = reinterpret_cast<const unsigned long long*>(p);
-  }
-  for (int m = 0; m < M; ++m)
-    for (int a = 0; a < 3; ++a) D.mdim[m][a] = mdim[m][a];
+  D.mdim0 = mdim[0];
+  D.mdim01 = mdim[0] * mdim[1];
   int2* dcells = nullptr;
   int32_t* dnodes = nullptr;
   int32_t* dorder = nullptr;
@@ -364,20 +298,6 @@ salf_status salf_build_scene_impl(salf_ctx* ctx, const salf_scene_desc* d, salf_
     if ((st = upload(s, box, &dbox)) != SALF_OK) return st;
     D.vox_box = dbox;
   }
-  for (int c = 0; c < CL; ++c) {
-    uint4* pc = nullptr;
-    if ((st = upload(s, cols[c], &pc)) != SALF_OK) return st;
-    D.col[c] = pc;
-    D.cdim[c][0] = cdim[c][0];
-    D.cdim[c][1] = cdim[c][1];
-  }
-  D.CL = CL;
-  {
-    int ls = 0;
-    while ((1 << ls) < layer_cells) ++ls;
-    D.layer_shift = ls + K;
-  }
-  D.n_layers = n_layers;
   void* status = nullptr;
   if ((st = dalloc(s, 16, &status)) != SALF_OK) return st;
   if ((ce = cudaMemset(status, 0, 16)) != cudaSuccess) return salf_cuda_fail(ce, "cudaMemset");
@@ -407,10 +327,10 @@ salf_status salf_build_scene_impl(salf_ctx* ctx, const salf_scene_desc* d, salf_
   if (n == 0)
     for (int a = 0; a < 3; ++a) D.bmin[a] = D.bmax[a] = 0;
   D.K = K;
-  D.M = M;
   D.mode = d->mode;
   D.dtype = d->dtype;
   D.n = (int)n;
+  if ((st = salf_build_skip(s, brick_p, brick_q, 0)) != SALF_OK) return st;
 
   if (n > 0) {
     const float* src = d->params;
@@ -439,6 +359,8 @@ salf_status salf_build_scene_impl(salf_ctx* ctx, const salf_scene_desc* d, salf_
       salf_set_error("salf_build_scene: SDF records need a > 0 and b > 0 (Eq. 6)");
       return SALF_ERR_INVALID;
     }
+  } else if ((ce = cudaDeviceSynchronize()) != cudaSuccess) {
+    return salf_cuda_fail(ce, "skip boxes");
   }
   guard.keep = true;
   *out = s;

@@ -78,8 +78,8 @@ __global__ void __launch_bounds__(256) k_secondary(const __grid_constant__ Secon
       c[k] = r.Oi[k] + (int)f;
       inside = inside && c[k] >= 0 && c[k] < S.Gf[k];
     }
-    int vox = -1, ls;
-    if (inside) vox = find_leaf(S, c[0], c[1], c[2], &ls);
+    int vox = -1, lx, lz;
+    if (inside) vox = find_leaf(S, c[0], c[1], c[2], &lx, &lz);
     float g[3] = {0.f, 0.f, 0.f};
     if (vox >= 0) record_slopes<DT>(S, vox, g);
     const float gg = g[0] * g[0] + g[1] * g[1] + g[2] * g[2];

@@ -9,14 +9,6 @@
 
 #include "salf_internal.h"
 
-// Traversal tuning switches (compile-time).
-#ifndef SALF_COL_MAX_LS
-#define SALF_COL_MAX_LS 0  // > 0: try the column skip only below this pyramid leaf size
-#endif
-#ifndef SALF_COL_EARLY
-#define SALF_COL_EARLY 1  // 1: load the column mask beside the pyramid word; 0: only for empty cells
-#endif
-
 namespace salf {
 
 constexpr float kPi = 3.14159265358979323846f;
@@ -166,79 +158,120 @@ __device__ __forceinline__ void dump_ray(const ReqDev& Q, const DevScene& S, con
   p[7] = r.valid ? 1.f : 0.f;
 }
 
-// Traversal state of one ray, all positions relative to the origin cell Oi so
-// that plane distances are small integers minus a fraction.
+// A ray's direction in finest cells per metre and its interval inside the
+// tight box of the voxels (no hit can lie outside it).  Zero direction
+// components become 1e-20.
+struct RayClip {
+  float D[3], invD[3];
+  float t0, t1;
+};
+
+__device__ __forceinline__ void ray_clip(const DevScene& S, const Ray& r, RayClip& q) {
+  const float isf = (float)S.inv_sfin;
+  q.t0 = r.tn;
+  q.t1 = r.tf;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    float D = r.d[a] * isf;
+    if (fabsf(D) < 1e-20f) D = 1e-20f;
+    q.D[a] = D;
+    q.invD[a] = 1.f / D;
+    const float lo = ((float)(S.bmin[a] - r.Oi[a]) - r.Of[a]) * q.invD[a];
+    const float hi = ((float)(S.bmax[a] - r.Oi[a]) - r.Of[a]) * q.invD[a];
+    q.t0 = fmaxf(q.t0, fminf(lo, hi));
+    q.t1 = fminf(q.t1, fmaxf(lo, hi));
+  }
+}
+
+// Traversal state of one ray.  Axes along which the ray travels downwards are
+// mirrored (plane p -> -p, cell c -> ~c, so the cell between planes c and c + 1
+// stays the one between its mirrored planes): every ray then travels upwards
+// on all three axes, a box is always left through its upper planes, and no
+// step selects planes by sign.  Mirroring negates both the plane offset
+// (p - Oi) - Of and 1 / D, so every distance is the unmirrored one bit for
+// bit.  Positions are relative to the origin cell Oi, so plane distances are
+// small integers minus a fraction.
 struct Walk {
-  int Oi[3];
-  float Of[3];
-  float D[3];     // direction in finest cells per metre (zero components -> 1e-20)
+  int Oi[3];      // origin cell, mirrored
+  float Of[3];    // origin inside it, mirrored
+  float D[3];     // |direction| in finest cells per metre
   float invD[3];  // metres per finest cell
-  int c[3];       // current finest cell
+  int r[3];       // current finest cell, mirrored, relative to Oi
+  unsigned neg;   // bit a: axis a is mirrored
+  const unsigned short* skip;  // skip boxes of the ray's octant, at mirrored brick (0, 0, 0)
   float t;        // entry distance of the current cell
-  float tend;     // min(t_far, root-box exit)
-  int steps;
-  int cl;         // column-pyramid level to try next
+  float tend;     // min(t_far, exit of the voxels' tight box)
   bool alive;
 };
+
+// 0 or all ones: axis a of the walk is mirrored.
+__device__ __forceinline__ int mirror_mask(const Walk& w, int a) {
+  return (int)(w.neg << (31 - a)) >> 31;
+}
+
+// x of a mirrored axis is -x.
+__device__ __forceinline__ float unmirror(const Walk& w, int a, float x) {
+  return __uint_as_float(__float_as_uint(x) ^ ((w.neg << (31 - a)) & 0x80000000u));
+}
 
 // (Re)start a walk at distance t: the cell holding the point there, kept
 // inside the tight box of the voxels.
 __device__ __forceinline__ void walk_seek(const DevScene& S, Walk& w, float t) {
   w.t = t;
-  w.steps = 0;
-  w.cl = min(S.CL - 1, 6);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    int q = w.Oi[a] + __float2int_rd(fmaf(t, w.D[a], w.Of[a]));
-    w.c[a] = min(max(q, S.bmin[a]), max(S.bmax[a] - 1, S.bmin[a]));
+    const int m = mirror_mask(w, a);
+    const int Oi = m ? -w.Oi[a] : w.Oi[a];
+    const int q = Oi + __float2int_rd(unmirror(w, a, fmaf(t, w.D[a], w.Of[a])));
+    w.r[a] = (min(max(q, S.bmin[a]), max(S.bmax[a] - 1, S.bmin[a])) ^ m) - w.Oi[a];
   }
 }
 
 __device__ __forceinline__ void walk_init(const DevScene& S, const Ray& r, Walk& w) {
-  float isf = (float)S.inv_sfin;
-  float t0 = r.tn, t1 = r.tf;
+  RayClip q;
+  ray_clip(S, r, q);
+  w.neg = 0u;
+  // the octant's skip boxes are stored in the mirrored brick order: brick b of
+  // axis a is entry b - base, mirrored n - 1 - (b - base) = ~b + base + n
+  long long off = 0, stride = 1;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    w.Oi[a] = r.Oi[a];
-    w.Of[a] = r.Of[a];
-    float D = r.d[a] * isf;
-    if (fabsf(D) < 1e-20f) D = 1e-20f;
-    w.D[a] = D;
-    w.invD[a] = 1.f / D;
-    // clip to the tight box of the voxels (no hit can lie outside it)
-    float lo = ((float)(S.bmin[a] - r.Oi[a]) - r.Of[a]) * w.invD[a];
-    float hi = ((float)(S.bmax[a] - r.Oi[a]) - r.Of[a]) * w.invD[a];
-    t0 = fmaxf(t0, fminf(lo, hi));
-    t1 = fminf(t1, fmaxf(lo, hi));
+    const bool neg = q.D[a] < 0.f;
+    w.neg |= neg ? 1u << a : 0u;
+    w.Oi[a] = neg ? -r.Oi[a] : r.Oi[a];
+    w.Of[a] = neg ? -r.Of[a] : r.Of[a];
+    w.D[a] = fabsf(q.D[a]);
+    w.invD[a] = fabsf(q.invD[a]);
+    off += stride * (neg ? S.skip_base[a] + S.skip_n[a] : -S.skip_base[a]);
+    stride *= S.skip_n[a];
   }
-  w.alive = r.valid && (t0 < t1);
-  w.tend = t1;
-  walk_seek(S, w, t0);
+  w.skip = S.skip + ((long long)w.neg * stride + off);
+  w.alive = r.valid && (q.t0 < q.t1);
+  w.tend = q.t1;
+  walk_seek(S, w, q.t0);
 }
 
 __device__ __forceinline__ void prefetch_l1(const void* p) {
   asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
 }
 
-__device__ __forceinline__ unsigned morton6(unsigned x, unsigned y, unsigned z) {
-  return (x & 1u) | ((y & 1u) << 1) | ((z & 1u) << 2) | ((x & 2u) << 2) | ((y & 2u) << 3) |
-         ((z & 2u) << 4);
-}
-
-// Leaf of the structure containing finest cell (ix, iy, iz): a voxel
-// (returns its internal index) or an empty region (returns -1).  *ls = log2 of
-// the leaf's edge in finest cells.
-__device__ __forceinline__ int find_leaf(const DevScene& S, int ix, int iy, int iz, int* ls) {
+// The voxel owning finest cell (ix, iy, iz), or -1 if the cell is empty.
+// *lx, *lz = log2 of the edges (x and y; z), in finest cells, of the aligned
+// box around the cell that lies in that voxel or is empty.
+__device__ __forceinline__ int find_leaf(const DevScene& S, int ix, int iy, int iz, int* lx,
+                                         int* lz) {
   const int K = S.K;
-  const unsigned cx = (unsigned)ix >> K, cy = (unsigned)iy >> K, cz = (unsigned)iz >> K;
-  const unsigned bx = cx >> 2, by = cy >> 2, bz = cz >> 2;
-  const uint4 w = __ldg(&S.mask0[(bz * (unsigned)S.mdim[0][1] + by) * (unsigned)S.mdim[0][0] + bx]);
-  const unsigned long long m = ((unsigned long long)w.y << 32) | (unsigned long long)w.x;
-  const unsigned bit = morton6(cx & 3, cy & 3, cz & 3);
-  if ((m >> bit) & 1ull) {
-    const unsigned pre = __popcll(m & ((1ull << bit) - 1ull));
+  const int cx = ix >> K, cy = iy >> K, cz = iz >> K;
+  const uint4 w = __ldg(&S.mask0[(unsigned)(cz >> 2) * (unsigned)S.mdim01 + (unsigned)(cy >> 2) * (unsigned)S.mdim0 + (unsigned)(cx >> 2)]);
+  // Morton bit of the cell inside its 4x4x4 block: z1 picks the word, then y1,
+  // x1, z0 the nibble of its 2x2x1 square, y0, x0 the bit
+  const unsigned half = (cz & 2) ? w.y : w.x;
+  const unsigned sh = ((cz & 1) << 2) | ((cx & 2) << 2) | ((cy & 2) << 3);
+  const unsigned bit = sh | (cx & 1) | ((cy & 1) << 1);
+  if ((half >> bit) & 1u) {
+    const unsigned pre = __popc(half & ((1u << bit) - 1u)) + ((cz & 2) ? __popc(w.x) : 0);
     if (w.w != 0xffffffffu) {  // block of level-0 voxels: no cell-table read
-      *ls = K;
+      *lx = *lz = K;
       return (int)(w.w + pre);
     }
     const int2 en = __ldg(&S.cells[w.z + pre]);
@@ -255,113 +288,19 @@ __device__ __forceinline__ int find_leaf(const DevScene& S, int ix, int iy, int 
       const int ch = ((ix >> l) & 1) | (((iy >> l) & 1) << 1) | (((iz >> l) & 1) << 2);
       e = __ldg(&S.nodes[(unsigned)(-2 - e) * 8u + (unsigned)ch]);
     }
-    *ls = l;
+    *lx = *lz = l;
     return e;
   }
-  if ((m >> (bit & 0x38u)) & 0xffull) {
-    *ls = K;
-    return -1;
-  }
-  if (m) {
-    *ls = K + 1;
-    return -1;
-  }
-  unsigned ux = bx, uy = by, uz = bz;
-  for (int lev = 1; lev < S.M; ++lev) {
-    const unsigned long long mw =
-        __ldg(&S.mask[lev][((uz >> 2) * (unsigned)S.mdim[lev][1] + (uy >> 2)) *
-                               (unsigned)S.mdim[lev][0] + (ux >> 2)]);
-    const unsigned b = morton6(ux & 3, uy & 3, uz & 3);
-    if ((mw >> (b & 0x38u)) & 0xffull) {
-      *ls = K + 2 * lev;
-      return -1;
-    }
-    if (mw) {
-      *ls = K + 2 * lev + 1;
-      return -1;
-    }
-    ux >>= 2;
-    uy >>= 2;
-    uz >>= 2;
-  }
-  *ls = K + 2 * S.M;
+  *lx = ((half >> sh) & 15u) ? K : K + 1;
+  *lz = K;
+  // bricks larger than a layer of a block (very large grids) may hold empty blocks
+  if (S.skip_coarse && !(w.x | w.y)) *lx = *lz = K + 2;
   return -1;
-}
-
-// Column-pyramid skip at level `cl` from the current (empty) cell: the ray may
-// advance through every layer of the 2^cl x 2^cl-column footprint that holds
-// no voxel, up to the nearest occupied layer in its direction of travel or the
-// footprint's side.  Returns false if the current layer is occupied in the
-// footprint (no progress at this level).  Fills the skipped box [lo, hi)
-// (finest cells), its exit axis and exit distance.
-// Column mask of the footprint (at level cl) that holds the current cell.
-__device__ __forceinline__ uint4 col_mask(const DevScene& S, const Walk& w, int cl) {
-  const int sh = S.K + cl;
-  return __ldg(&S.col[cl][(unsigned)(w.c[1] >> sh) * (unsigned)S.cdim[cl][0] +
-                          (unsigned)(w.c[0] >> sh)]);
-}
-
-__device__ __forceinline__ bool col_skip(const DevScene& S, const Walk& w, int cl, const uint4 m,
-                                         float* t_exit, int lo[3], int hi[3], int* axis) {
-  const int sh = S.K + cl;
-  const int F = 1 << sh;
-  const int fx = w.c[0] >> sh, fy = w.c[1] >> sh;
-  const int bx = fx << sh, by = fy << sh;
-  const float tx = ((float)((w.D[0] > 0.f ? bx + F : bx) - w.Oi[0]) - w.Of[0]) * w.invD[0];
-  const float ty = ((float)((w.D[1] > 0.f ? by + F : by) - w.Oi[1]) - w.Of[1]) * w.invD[1];
-  float te = fminf(tx, ty);
-  int ax = tx <= ty ? 0 : 1;
-  const bool up = w.D[2] > 0.f;
-  const int LS = S.layer_shift;
-  const int lcur = w.c[2] >> LS;
-  // furthest layer the ray reaches inside the footprint (widened toward travel)
-  const float zf = (float)w.Oi[2] + fmaf(fminf(te, w.tend), w.D[2], w.Of[2]) + (up ? 1e-3f : -1e-3f);
-  int lend = __float2int_rd(zf) >> LS;
-  lend = min(max(lend, 0), S.n_layers - 1);
-  const unsigned long long lo64 = ((unsigned long long)m.y << 32) | m.x;
-  const unsigned long long hi64 = ((unsigned long long)m.w << 32) | m.z;
-  int Ls;  // nearest occupied layer at or beyond lcur in the direction of travel
-  if (up) {
-    const unsigned long long a = lcur < 64 ? (lo64 & (~0ull << lcur)) : 0ull;
-    const unsigned long long b = lcur < 64 ? hi64 : (hi64 & (~0ull << (lcur - 64)));
-    Ls = a ? (__ffsll((long long)a) - 1) : (b ? (63 + __ffsll((long long)b)) : 1 << 20);
-  } else {
-    const unsigned long long a = lcur >= 64 ? lo64 : (lo64 & ((2ull << lcur) - 1ull));
-    const unsigned long long b = lcur >= 64 ? (hi64 & ((2ull << (lcur - 64)) - 1ull)) : 0ull;
-    Ls = b ? (127 - __clzll((long long)b)) : (a ? (63 - __clzll((long long)a)) : -(1 << 20));
-  }
-  if (Ls == lcur) return false;
-  const bool reach = up ? (Ls <= lend) : (Ls >= lend);
-  int zlo, zhi;
-  if (up) {
-    zlo = lcur << LS;
-    zhi = (reach ? Ls : lend + 1) << LS;
-  } else {
-    zlo = (reach ? Ls + 1 : lend) << LS;
-    zhi = (lcur + 1) << LS;
-  }
-  if (reach) {
-    const int zb = up ? zlo + (zhi - zlo) : zlo;  // boundary plane of layer Ls facing the ray
-    const float tz = ((float)(zb - w.Oi[2]) - w.Of[2]) * w.invD[2];
-    if (tz < te) {
-      te = tz;
-      ax = 2;
-    }
-  }
-  lo[0] = bx;
-  hi[0] = bx + F;
-  lo[1] = by;
-  hi[1] = by + F;
-  lo[2] = zlo;
-  hi[2] = zhi;
-  *axis = ax;
-  *t_exit = te;
-  return te > w.t;
 }
 
 struct Hit {
   int vox;
-  int base[3];
+  int lo[3];  // min corner, mirrored, relative to the origin cell
   int ls;
   float tin, tout;
 };
@@ -370,43 +309,10 @@ struct Hit {
 // from the start began): the same formula as the entry next_hit reports, but
 // independent of where a walk started, so every walk of one ray agrees on it.
 __device__ __forceinline__ float hit_entry(const Walk& w, const Hit& h, float t0) {
-  const int E = 1 << h.ls;
   float t = t0;
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const int p = (w.D[a] > 0.f ? h.base[a] : h.base[a] + E) - w.Oi[a];
-    t = fmaxf(t, ((float)p - w.Of[a]) * w.invD[a]);
-  }
+  for (int a = 0; a < 3; ++a) t = fmaxf(t, ((float)h.lo[a] - w.Of[a]) * w.invD[a]);
   return t;
-}
-
-// Leave the box [lo, hi) through its face on `axis` at distance te: the next
-// point to locate is the neighbour cell across that face, the other
-// coordinates taken from the exit point, kept inside the box's face and never
-// moved backwards (so every hop makes progress).
-__device__ __forceinline__ void hop(const DevScene& S, Walk& w, const int lo[3], const int hi[3],
-                                    int axis, float te) {
-  if (!(te < w.tend) || ++w.steps > S.Gf[0] + S.Gf[1] + S.Gf[2] + 64) {
-    if (w.steps > S.Gf[0] + S.Gf[1] + S.Gf[2] + 64) atomicOr(S.status, SALF_DEVERR_STEP_CAP);
-    w.alive = false;
-    return;
-  }
-  bool out = false;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    if (a == axis) {
-      const int n = w.D[a] > 0.f ? hi[a] : lo[a] - 1;
-      out = n < 0 || n >= S.Gf[a];
-      w.c[a] = n;
-    } else {
-      int q = w.Oi[a] + __float2int_rd(fmaf(te, w.D[a], w.Of[a]));
-      q = min(max(q, lo[a]), hi[a] - 1);
-      q = min(q, S.Gf[a] - 1);  // boxes start at >= 0, so q >= 0 already
-      w.c[a] = w.D[a] > 0.f ? max(q, w.c[a]) : min(q, w.c[a]);
-    }
-  }
-  if (out) w.alive = false;
-  w.t = fmaxf(w.t, te);
 }
 
 // Advance `w` by one structure step toward the next voxel crossed with
@@ -414,86 +320,73 @@ __device__ __forceinline__ void hop(const DevScene& S, Walk& w, const int lo[3],
 // composites the lanes that found one, then calls again: one step per call
 // keeps lanes of different rays in step, so a warp costs about its heaviest
 // ray, not the sum of per-round maxima (two or three steps per call measured
-// slower, and the loop for them cost 1-3% even when it ran once).  Empty space
-// is left through the farther of two empty boxes around the current cell: the
-// largest empty aligned pyramid cell, and the column-pyramid skip.
-// FMIN: take the exit distance as the minimum of the three plane distances
-// (the same value as indexing them by the exit axis, as they are finite); the
-// indexed form keeps the array in local memory, the minimum does not.  The
-// span-parallel kernel measured 1.3% slower with it, so it keeps the indexed
-// form.
-template <bool FMIN = true>
+// slower, and the loop for them cost 1-3% even when it ran once).
+//
+// A step reads the skip box of the current brick for the ray's octant (2
+// bytes).  An empty brick's box reaches up to 31 x 31 x 63 bricks ahead in the
+// ray's own directions; a brick that holds voxels has no box, and the cell is
+// located in its block (find_leaf).  Either way the box is left through its
+// nearest upper plane; the other coordinates come from the exit point, kept
+// inside the box and never moved backwards.
+//
+// Every step ends inside the skip array: boxes end inside it, the start is
+// inside the tight box, and a ray whose exit plane is not before the tight
+// box's (te >= tend) takes no further step.  The exit axis always advances, so
+// a walk ends after at most the array's cells per axis.
 __device__ __forceinline__ bool next_hit(const DevScene& S, Walk& w, Hit& h) {
-  if (w.alive) {
-    // the column mask depends only on the cell: issue its load with the pyramid's
-    const int cl = w.cl;
-#if SALF_COL_EARLY
-    const uint4 cmask = col_mask(S, w, cl);
-#endif
-    int ls;
-    const int vox = find_leaf(S, w.c[0], w.c[1], w.c[2], &ls);
-    const int E = 1 << ls;
-    int lo[3], hi[3];
-    float tx[3];
+  if (!w.alive) return false;
+  int c[3], b[3], e[3], rel[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) c[a] = w.r[a] + w.Oi[a];
+  int sx = S.skip_sx, sz = S.skip_sz;
+  b[0] = c[0] >> sx;
+  b[1] = c[1] >> sx;
+  b[2] = c[2] >> sz;
+  const unsigned v = __ldg(w.skip + ((long long)b[2] * S.skip_n01 + (b[1] * S.skip_n[0] + b[0])));
+  e[0] = v & 31u;
+  e[1] = (v >> 5) & 31u;
+  e[2] = v >> 10;
+  int vox = -1;
+  if (v == 0u) {
+    vox = find_leaf(S, c[0] ^ mirror_mask(w, 0), c[1] ^ mirror_mask(w, 1),
+                    c[2] ^ mirror_mask(w, 2), &sx, &sz);
+    b[0] = c[0] >> sx;
+    b[1] = c[1] >> sx;
+    b[2] = c[2] >> sz;
+    e[0] = e[1] = e[2] = 1;
+  }
+  float tx[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    rel[a] = ((b[a] + e[a]) << (a == 2 ? sz : sx)) - w.Oi[a];
+    tx[a] = ((float)rel[a] - w.Of[a]) * w.invD[a];
+  }
+  const float te = fminf(fminf(tx[0], tx[1]), tx[2]);
+  bool found = false;
+  if (vox >= 0) {
+    float tin = w.t;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      lo[a] = w.c[a] & ~(E - 1);
-      hi[a] = lo[a] + E;
-      const int p = (w.D[a] > 0.f ? hi[a] : lo[a]) - w.Oi[a];
-      tx[a] = ((float)p - w.Of[a]) * w.invD[a];
+      h.lo[a] = rel[a] - (1 << sx);
+      tin = fmaxf(tin, ((float)h.lo[a] - w.Of[a]) * w.invD[a]);
     }
-    int ax = (tx[0] <= tx[1] && tx[0] <= tx[2]) ? 0 : (tx[1] <= tx[2] ? 1 : 2);
-    float te = FMIN ? fminf(fminf(tx[0], tx[1]), tx[2]) : tx[ax];
-    bool found = false;
-    if (vox >= 0) {
-      float tin = w.t;
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        const int p = (w.D[a] > 0.f ? lo[a] : hi[a]) - w.Oi[a];
-        tin = fmaxf(tin, ((float)p - w.Of[a]) * w.invD[a]);
-      }
-      const float tout = fminf(te, w.tend);
-      found = tout > tin;
-      // start fetching the voxel's record: it is read right after this step
-      prefetch_l1(static_cast<const char*>(S.params) +
-                  (size_t)vox * (S.dtype == SALF_F32 ? 128u : 64u));
-      h.vox = vox;
-      h.ls = ls;
-      h.base[0] = lo[0];
-      h.base[1] = lo[1];
-      h.base[2] = lo[2];
-      h.tin = tin;
-      h.tout = tout;
-    } else {
-      // empty: the column-pyramid skip replaces the pyramid cell if it goes further
-      int clo[3], chi[3], cax;
-      float cte;
-      bool ok = false;
-#if SALF_COL_MAX_LS > 0
-      if (ls <= SALF_COL_MAX_LS + S.K)
-#endif
-      {
-#if !SALF_COL_EARLY
-        const uint4 cmask = col_mask(S, w, cl);
-#endif
-        ok = col_skip(S, w, cl, cmask, &cte, clo, chi, &cax);
-        w.cl = ok ? min(cl + 1, S.CL - 1) : max(cl - 1, 0);
-      }
-      if (ok && cte > te) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          lo[a] = clo[a];
-          hi[a] = chi[a];
-        }
-        ax = cax;
-        te = cte;
-      }
-    }
-    // one hop for every lane, whichever box it leaves (keeps the warp converged)
-    hop(S, w, lo, hi, ax, te);
-    return found;
+    h.tin = tin;
+    h.tout = fminf(te, w.tend);
+    found = h.tout > tin;
+    h.vox = vox;
+    h.ls = sx;
+    // start fetching the voxel's record: it is read right after this step
+    prefetch_l1(static_cast<const char*>(S.params) +
+                (size_t)vox * (S.dtype == SALF_F32 ? 128u : 64u));
   }
-  return false;
+  w.alive = te < w.tend;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int q = max(w.r[a], min(__float2int_rd(fmaf(te, w.D[a], w.Of[a])), rel[a] - 1));
+    w.r[a] = tx[a] <= te ? rel[a] : q;
+  }
+  w.t = fmaxf(w.t, te);
+  return found;
 }
 
 // ---------------------------------------------------------------- records
@@ -533,16 +426,16 @@ struct Record<SALF_BF16> {
   }
 };
 
-// Local coordinates of the segment midpoint inside the voxel box
-// [base, base + 2^ls) (finest cells): x = (p - centre) / (edge / 2).
+// Local coordinates of the segment midpoint (distance tm) inside a hit's box:
+// x = (p - centre) / (edge / 2).
 __device__ __forceinline__ void local_coords(const Walk& w, const Hit& h, float tm, float x[3]) {
   const float E = (float)(1 << h.ls);
   const float inv_half = __int_as_float((128 - h.ls) << 23);  // 2 / E, exact: E = 2^ls
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    float p = fmaf(tm, w.D[a], w.Of[a]);  // relative to the origin cell
-    float ctr = (float)(h.base[a] - w.Oi[a]) + 0.5f * E;
-    x[a] = (p - ctr) * inv_half;
+    const float p = fmaf(tm, w.D[a], w.Of[a]);  // relative to the origin cell
+    const float ctr = (float)h.lo[a] + 0.5f * E;
+    x[a] = unmirror(w, a, (p - ctr) * inv_half);
   }
 }
 
@@ -695,18 +588,14 @@ struct Accum {
   float Rp;  // sum of T_i alpha_i sigmoid(rho_i) (raydrop, when asked for)
 };
 
-// Composite one hit voxel with its field at the segment midpoint: alpha =
-// 1 - exp(-sigma delta) (Eq. 4), weight T alpha (Eq. 3).  The ray kernel and
-// the tile rasteriser both call this, so their arithmetic is the same.
-// Returns 1 - alpha.
+// Composite one hit voxel of length dl with its field at the segment midpoint
+// (distance tm, local coordinates x): alpha = 1 - exp(-sigma delta) (Eq. 4),
+// weight T alpha (Eq. 3).  The ray kernel and the tile rasteriser both call
+// this, so their arithmetic is the same.  Returns 1 - alpha.
 template <int DT, int MODE, class Src>
-__device__ __forceinline__ float composite_hit(const Walk& w, const Hit& h, const Src& src,
-                                              bool want_int, const float gam[4], Accum& A,
-                                              bool want_drop = false) {
-  const float tm = 0.5f * (h.tin + h.tout);
-  const float dl = h.tout - h.tin;
-  float x[3];
-  local_coords(w, h, tm, x);
+__device__ __forceinline__ float composite_at(const float x[3], float tm, float dl, const Src& src,
+                                             bool want_int, const float gam[4], Accum& A,
+                                             bool want_drop = false) {
   Field f;
   field_eval_src<DT, MODE>(src, want_int, x, gam, f, want_drop);
   const float e = __expf(-f.sig * dl);  // 1 - alpha (Eq. 4)
@@ -719,6 +608,16 @@ __device__ __forceinline__ float composite_hit(const Walk& w, const Hit& h, cons
   if (want_drop) A.Rp = fmaf(wgt, f.dr, A.Rp);
   A.T *= e;
   return e;
+}
+
+template <int DT, int MODE, class Src>
+__device__ __forceinline__ float composite_hit(const Walk& w, const Hit& h, const Src& src,
+                                              bool want_int, const float gam[4], Accum& A,
+                                              bool want_drop = false) {
+  const float tm = 0.5f * (h.tin + h.tout);
+  float x[3];
+  local_coords(w, h, tm, x);
+  return composite_at<DT, MODE>(x, tm, h.tout - h.tin, src, want_int, gam, A, want_drop);
 }
 
 // Per-ray outputs of a request (colour premultiplied, background added with

@@ -328,14 +328,14 @@ __global__ void __launch_bounds__(32 * kActorWarps,
     const bool start_next =
         cur < 0 && nxt < ni && (!hs_ok || nxt_in <= hs.tin + 1e-5f * fmaxf(1.f, fabsf(hs.tin)));
     if (!hs_ok && ws.alive) {
-      hs_ok = next_hit(S, ws, hs);
+      hs_ok = next_hit<DT>(S, ws, hs);
     } else if (start_next) {
       cur = iv_k[nxt++];
       nxt_in = nxt < ni ? iv_in[nxt] : 0.f;
       actor_walk(actors[cur], r, wa, gam_a);
       ha_ok = false;
     } else if (cur >= 0 && !ha_ok && wa.alive) {
-      ha_ok = next_hit(actors[cur].S, wa, ha);
+      ha_ok = next_hit<DT>(actors[cur].S, wa, ha);
     }
     // an actor walk that ended this round (or opened empty) leaves the next
     // interval to be weighed against the pending static hit
@@ -553,7 +553,7 @@ __global__ void __launch_bounds__(32 * kActorWarps, SALF_ACTOR_MIN_BLOCKS) k_bac
     const bool start_next =
         cur < 0 && nxt < ni && (!hs_ok || nxt_in <= hs.tin + 1e-5f * fmaxf(1.f, fabsf(hs.tin)));
     if (!hs_ok && ws.alive) {
-      hs_ok = next_hit(S, ws, hs);
+      hs_ok = next_hit<DT>(S, ws, hs);
     } else if (start_next) {
       cur = iv_k[nxt++];
       nxt_in = nxt < ni ? iv_in[nxt] : 0.f;
@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(32 * kActorWarps, SALF_ACTOR_MIN_BLOCKS) k_bac
       actor_walk(actors[cur], r, wa, gam_a);
       ha_ok = false;
     } else if (cur >= 0 && !ha_ok && wa.alive) {
-      ha_ok = next_hit(actors[cur].S, wa, ha);
+      ha_ok = next_hit<DT>(actors[cur].S, wa, ha);
     }
     // an actor walk that ended this round (or opened empty) leaves the next
     // interval to be weighed against the pending static hit

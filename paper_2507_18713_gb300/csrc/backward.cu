@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(32 * SALF_BWD_WARPS, SALF_BWD_MIN_BLOCKS)
 
   for (;;) {
     Hit h;
-    const bool hit = next_hit(S, w, h);
+    const bool hit = next_hit<DT>(S, w, h);
     if (!__any_sync(0xffffffffu, hit || w.alive)) break;
     const unsigned hit_lanes = __ballot_sync(0xffffffffu, hit);
     if (hit) {

@@ -29,9 +29,10 @@
 
 // Warps per block and resident blocks per SM of each forward variant (they
 // bound the registers per thread).  Coherent camera batches are throughput-
-// bound and gain from more resident warps; divergent sensors (fisheye,
-// panorama, LiDAR) are bound by their heaviest warps' latency and lose more to
-// the register spills that extra residency costs.
+// bound and gain from more resident warps (7 blocks: 1080p camera 265 us; 6
+// blocks 277, 8 blocks 279, with spills).  Divergent sensors (fisheye,
+// panorama, LiDAR) take 20 warps per SM (96 registers): LiDAR 237 us, fisheye
+// 298; 16 warps 282 / 301, 24 warps 264 / 301, 28 warps (fisheye) 340.
 #ifndef SALF_FWD_WPB_COHERENT
 #define SALF_FWD_WPB_COHERENT 4
 #endif
@@ -43,17 +44,17 @@
 #define SALF_FWD_COHERENT_KINDS ((1 << SALF_PINHOLE) | (1 << SALF_RAYS_EXPLICIT))
 #endif
 #ifndef SALF_FWD_WPB_DIVERGENT
-#define SALF_FWD_WPB_DIVERGENT 8
+#define SALF_FWD_WPB_DIVERGENT 4
 #endif
 #ifndef SALF_FWD_BLOCKS_DIVERGENT
-#define SALF_FWD_BLOCKS_DIVERGENT 2
+#define SALF_FWD_BLOCKS_DIVERGENT 5
 #endif
 // Span-parallel variant (batches with a request of more than one span per ray).
 #ifndef SALF_FWD_WPB_SEG
-#define SALF_FWD_WPB_SEG 8
+#define SALF_FWD_WPB_SEG 4
 #endif
 #ifndef SALF_FWD_BLOCKS_SEG
-#define SALF_FWD_BLOCKS_SEG 2
+#define SALF_FWD_BLOCKS_SEG 5
 #endif
 
 using namespace salf;
@@ -133,7 +134,7 @@ __global__ void __launch_bounds__(32 * WPB, MINB) k_forward(const __grid_constan
     for (;;) {
       Hit h;
       if (DUMP) steps += w.alive ? 1 : 0;
-      bool hit = next_hit(S, w, h);
+      bool hit = next_hit<DT>(S, w, h);
       if (SEG && !hit && w.t > walk_end) w.alive = false;  // the rest is the next span's
       if (!__any_sync(0xffffffffu, hit || w.alive)) break;
       if (SEG && hit && ks > 0) {  // composite only the voxels entered inside this span

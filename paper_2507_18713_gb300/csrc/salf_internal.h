@@ -66,11 +66,11 @@ struct DevScene {
   int mdim0, mdim01;  // blocks per row (x) and per layer (x, y)
   const int2* cells;
   const int* nodes;
-  // octant o (bit a: the ray travels downwards on axis a) starts at
-  // o * skip_n01 * skip_n[2], bricks in mirrored order on its downward axes
-  const unsigned short* skip;
-  int skip_n[3], skip_n01;  // bricks per axis; per layer
-  int skip_base[3];         // first brick per axis (brick = cell >> shift)
+  // skip boxes of octant o (bit a: the ray travels downwards on axis a), bricks in
+  // mirrored order on its downward axes, moved so that the index is the (mirrored)
+  // brick's own: b2 * skip_n01 + b1 * skip_n0 + b0
+  const unsigned short* skip_oct[8];
+  int skip_n0, skip_n01;    // bricks per row (x) and per layer (x, y)
   int skip_sx, skip_sz;     // log2 of a brick's edges (x and y; z), finest cells
   int skip_coarse;          // bricks are larger than a layer of a block
   const void* params;

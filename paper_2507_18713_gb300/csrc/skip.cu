@@ -248,11 +248,18 @@ salf_status salf_build_skip(salf_scene* s, int p, int q, cudaStream_t st) {
       rect, G, tiles_x, static_cast<unsigned short*>(skip));
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return salf_cuda_fail(e, "skip boxes");
-  D.skip = static_cast<const unsigned short*>(skip);
-  for (int a = 0; a < 3; ++a) {
-    D.skip_n[a] = G.n[a];
-    D.skip_base[a] = G.base[a];
+  // brick b of axis a is entry b - base of an octant, mirrored (~b) entry
+  // n - 1 - (b - base) = ~b + base + n
+  for (int o = 0; o < 8; ++o) {
+    long long off = o * n01 * G.n[2], stride = 1;
+    for (int a = 0; a < 3; ++a) {
+      off += stride * ((o >> a) & 1 ? G.base[a] + G.n[a] : -G.base[a]);
+      stride *= G.n[a];
+    }
+    D.skip_oct[o] = reinterpret_cast<const unsigned short*>(
+        reinterpret_cast<uintptr_t>(skip) + (uintptr_t)(off * (long long)sizeof(unsigned short)));
   }
+  D.skip_n0 = G.n[0];
   D.skip_n01 = (int)n01;
   D.skip_sx = D.K + p;
   D.skip_sz = D.K + q;

@@ -231,9 +231,6 @@ __device__ __forceinline__ void walk_init(const DevScene& S, const Ray& r, Walk&
   RayClip q;
   ray_clip(S, r, q);
   w.neg = 0u;
-  // the octant's skip boxes are stored in the mirrored brick order: brick b of
-  // axis a is entry b - base, mirrored n - 1 - (b - base) = ~b + base + n
-  long long off = 0, stride = 1;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const bool neg = q.D[a] < 0.f;
@@ -242,10 +239,8 @@ __device__ __forceinline__ void walk_init(const DevScene& S, const Ray& r, Walk&
     w.Of[a] = neg ? -r.Of[a] : r.Of[a];
     w.D[a] = fabsf(q.D[a]);
     w.invD[a] = fabsf(q.invD[a]);
-    off += stride * (neg ? S.skip_base[a] + S.skip_n[a] : -S.skip_base[a]);
-    stride *= S.skip_n[a];
   }
-  w.skip = S.skip + ((long long)w.neg * stride + off);
+  w.skip = S.skip_oct[w.neg];
   w.alive = r.valid && (q.t0 < q.t1);
   w.tend = q.t1;
   walk_seek(S, w, q.t0);
@@ -333,6 +328,7 @@ __device__ __forceinline__ float hit_entry(const Walk& w, const Hit& h, float t0
 // inside the tight box, and a ray whose exit plane is not before the tight
 // box's (te >= tend) takes no further step.  The exit axis always advances, so
 // a walk ends after at most the array's cells per axis.
+template <int DT>
 __device__ __forceinline__ bool next_hit(const DevScene& S, Walk& w, Hit& h) {
   if (!w.alive) return false;
   int c[3], b[3], e[3], rel[3];
@@ -342,7 +338,7 @@ __device__ __forceinline__ bool next_hit(const DevScene& S, Walk& w, Hit& h) {
   b[0] = c[0] >> sx;
   b[1] = c[1] >> sx;
   b[2] = c[2] >> sz;
-  const unsigned v = __ldg(w.skip + ((long long)b[2] * S.skip_n01 + (b[1] * S.skip_n[0] + b[0])));
+  const unsigned v = __ldg(w.skip + ((long long)b[2] * S.skip_n01 + (b[1] * S.skip_n0 + b[0])));
   e[0] = v & 31u;
   e[1] = (v >> 5) & 31u;
   e[2] = v >> 10;
@@ -377,12 +373,12 @@ __device__ __forceinline__ bool next_hit(const DevScene& S, Walk& w, Hit& h) {
     h.ls = sx;
     // start fetching the voxel's record: it is read right after this step
     prefetch_l1(static_cast<const char*>(S.params) +
-                (size_t)vox * (S.dtype == SALF_F32 ? 128u : 64u));
+                (size_t)vox * (DT == SALF_F32 ? 128u : 64u));
   }
   w.alive = te < w.tend;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const int q = max(w.r[a], min(__float2int_rd(fmaf(te, w.D[a], w.Of[a])), rel[a] - 1));
+    const int q = max(w.r[a], __viaddmin_s32(rel[a], -1, __float2int_rd(fmaf(te, w.D[a], w.Of[a]))));
     w.r[a] = tx[a] <= te ? rel[a] : q;
   }
   w.t = fmaxf(w.t, te);

@@ -6,7 +6,7 @@
 // split threshold becomes its 8 octree children; the rest are kept.  An
 // exclusive scan of the output counts (0, 8 or 1) places every voxel's
 // output in input order, children in place of their parent.
-// Apply (one thread per voxel): writes level, cell and record of each output
+// Apply (8 lanes per voxel): writes level, cell and record of each output
 // voxel.  A child's record carries its parent's fields exactly: every field
 // is affine in the local coordinates and x_parent = (x_child + o) / 2 with
 // o in {-1, +1}^3, so the slopes halve and the offsets take W . o / 2 (the
@@ -24,16 +24,18 @@ namespace {
 
 constexpr float kSH0 = 0.28209479177387814f;
 
+// In input order, from the scene's keys: neighbouring threads read neighbouring
+// rows; the counts are summed over a block before their atomics (1M voxels: 27 us;
+// in voxel order with an atomic per warp and count 57).
 __global__ void __launch_bounds__(256) k_refine_plan(
-    const int4* __restrict__ vox_box, const int* __restrict__ order, int n, int K,
-    const float* __restrict__ grads, const float* __restrict__ max_alpha, float split_thr,
-    float prune_alpha, unsigned char* __restrict__ action, unsigned* __restrict__ count,
+    const uint8_t* __restrict__ key_level, int n, int K, const float* __restrict__ grads,
+    const float* __restrict__ max_alpha, float split_thr, float prune_alpha,
+    unsigned char* __restrict__ action, unsigned* __restrict__ count,
     unsigned long long* __restrict__ stats) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  const int v = blockIdx.x * blockDim.x + threadIdx.x;
   int act = -1;
-  if (p < n) {
-    const int v = __ldg(&order[p]);
-    const int level = K - __ldg(&vox_box[p]).w;
+  if (v < n) {
+    const int level = __ldg(&key_level[v]);
     const float4* g = reinterpret_cast<const float4*>(grads) + (size_t)v * 8;
     const float4 g1 = __ldg(g + 1), g2 = __ldg(g + 2), g3 = __ldg(g + 3);  // slots 4..15
     const float l1 = fabsf(g1.x) + fabsf(g1.y) + fabsf(g1.z) + fabsf(g1.w) + fabsf(g2.x) +
@@ -45,72 +47,87 @@ __global__ void __launch_bounds__(256) k_refine_plan(
   }
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const unsigned c = __reduce_add_sync(0xffffffffu, act == k ? 1u : 0u);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd(&stats[k], (unsigned long long)c);
+    const int c = __syncthreads_count(act == k);
+    if (threadIdx.x == 0 && c) atomicAdd(&stats[k], (unsigned long long)c);
   }
 }
 
+// 8 lanes per voxel, a 16-byte chunk of the record each, so that every row is
+// read and written as one 128-byte line; kRows voxels per group, whose loads are
+// in flight together.  A child's chunk needs other chunks' colour rows and
+// intensity slopes: shuffles inside the 8 lanes; all lanes run the same code (a
+// switch over the chunks cost as much as the scattered rows saved).  1M voxels
+// in, 1.27M out (310 MB): 59 us; a thread per voxel 101.
+constexpr int kRows = 4;
+
 __global__ void __launch_bounds__(256) k_refine_apply(
-    const int4* __restrict__ vox_box, const int* __restrict__ order, int n, int K,
+    const uint8_t* __restrict__ key_level, const int* __restrict__ key_ijk, int n,
     const unsigned char* __restrict__ action, const unsigned long long* __restrict__ offs,
     const float* __restrict__ params, unsigned char* __restrict__ level_out,
     int* __restrict__ ijk_out, float* __restrict__ params_out) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  const int v = __ldg(&order[p]);
-  const int act = __ldg(&action[v]);
-  if (act == 2) return;
-  const int4 b = __ldg(&vox_box[p]);
-  const int level = K - b.w;
-  const int ijk[3] = {b.x >> b.w, b.y >> b.w, b.z >> b.w};
-  float rec[32];
-  const float4* src = reinterpret_cast<const float4*>(params) + (size_t)v * 8;
+  const int k = (int)(threadIdx.x & 7);  // chunk: slots 4 k .. 4 k + 3
+  const long long v0 = blockIdx.x * (32LL * kRows) + (threadIdx.x >> 3);
+  int act[kRows], level[kRows], cell[kRows];  // cell: axis k of ijk on lanes 0..2
+  unsigned long long o[kRows];
+  float4 rec[kRows];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const float4 q = __ldg(src + k);
-    rec[4 * k] = q.x;
-    rec[4 * k + 1] = q.y;
-    rec[4 * k + 2] = q.z;
-    rec[4 * k + 3] = q.w;
-  }
-  const unsigned long long o = __ldg(&offs[v]);
-  if (act == 0) {
-    level_out[o] = (unsigned char)level;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) ijk_out[3 * o + a] = ijk[a];
-    float4* dst = reinterpret_cast<float4*>(params_out) + (size_t)o * 8;
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      dst[k] = make_float4(rec[4 * k], rec[4 * k + 1], rec[4 * k + 2], rec[4 * k + 3]);
-    return;
-  }
-  for (int c = 0; c < 8; ++c) {
-    const float s[3] = {(c & 1) ? 1.f : -1.f, (c & 2) ? 1.f : -1.f, (c & 4) ? 1.f : -1.f};
-    float out[32];
-#pragma unroll
-    for (int k = 0; k < 32; ++k) out[k] = rec[k];
-    out[3] = rec[3] + 0.5f * (rec[0] * s[0] + rec[1] * s[1] + rec[2] * s[2]);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) out[a] = 0.5f * rec[a];
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-      const float shift = rec[4 + 3 * r] * s[0] + rec[5 + 3 * r] * s[1] + rec[6 + 3 * r] * s[2];
-#pragma unroll
-      for (int a = 0; a < 3; ++a) out[4 + 3 * r + a] = 0.5f * rec[4 + 3 * r + a];
-      out[13 + 4 * r] = rec[13 + 4 * r] + 0.5f * shift / kSH0;
+  for (int j = 0; j < kRows; ++j) {
+    const long long v = v0 + 32 * j;
+    act[j] = v < n ? __ldg(&action[v]) : 2;
+    rec[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+    o[j] = 0;
+    level[j] = cell[j] = 0;
+    if (v < n) {
+      rec[j] = __ldg(reinterpret_cast<const float4*>(params) + v * 8 + k);
+      o[j] = __ldg(&offs[v]);
+      level[j] = __ldg(&key_level[v]);
+      if (k < 3) cell[j] = __ldg(&key_ijk[3 * v + k]);
     }
-    out[30] = rec[30] + 0.5f * (rec[27] * s[0] + rec[28] * s[1] + rec[29] * s[2]);
+  }
 #pragma unroll
-    for (int a = 0; a < 3; ++a) out[27 + a] = 0.5f * rec[27 + a];
-    const unsigned long long oc = o + (unsigned long long)c;
-    level_out[oc] = (unsigned char)(level + 1);
-    ijk_out[3 * oc] = 2 * ijk[0] + (c & 1);
-    ijk_out[3 * oc + 1] = 2 * ijk[1] + ((c >> 1) & 1);
-    ijk_out[3 * oc + 2] = 2 * ijk[2] + ((c >> 2) & 1);
-    float4* dst = reinterpret_cast<float4*>(params_out) + (size_t)oc * 8;
+  for (int j = 0; j < kRows; ++j) {
+    const float4 q = rec[j];
+    float4* dst = reinterpret_cast<float4*>(params_out) + (size_t)o[j] * 8 + k;
+    if (act[j] == 0) {
+      *dst = q;
+      if (k == 0) level_out[o[j]] = (unsigned char)level[j];
+      if (k < 3) ijk_out[3 * o[j] + k] = cell[j];
+    }
+    if (!__any_sync(0xffffffffu, act[j] == 1)) continue;
+    const unsigned full = 0xffffffffu;
+    const int ijk[3] = {__shfl_sync(full, cell[j], 0, 8), __shfl_sync(full, cell[j], 1, 8),
+                        __shfl_sync(full, cell[j], 2, 8)};
+    // slots 4..12 (colour rows) and 27 for every lane of the voxel
+    const float c4 = __shfl_sync(full, q.x, 1, 8), c5 = __shfl_sync(full, q.y, 1, 8),
+                c6 = __shfl_sync(full, q.z, 1, 8), c7 = __shfl_sync(full, q.w, 1, 8),
+                c8 = __shfl_sync(full, q.x, 2, 8), c9 = __shfl_sync(full, q.y, 2, 8),
+                c10 = __shfl_sync(full, q.z, 2, 8), c11 = __shfl_sync(full, q.w, 2, 8),
+                c12 = __shfl_sync(full, q.x, 3, 8), c27 = __shfl_sync(full, q.w, 6, 8);
+    if (act[j] != 1) continue;
+    level_out[o[j] + k] = (unsigned char)(level[j] + 1);
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
-      dst[k] = make_float4(out[4 * k], out[4 * k + 1], out[4 * k + 2], out[4 * k + 3]);
+    for (int a = 0; a < 3; ++a) ijk_out[3 * (o[j] + k) + a] = 2 * ijk[a] + ((k >> a) & 1);
+    // slopes halve (hx..hw), and one component of the chunk moves by half of
+    // (A, B, C) . s, over C0 where it is an SH DC term
+    const bool sh = k >= 3 && k <= 5;
+    const float A = k == 0 ? q.x : (k == 3 ? c4 : (k == 4 ? c7 : (k == 5 ? c10 : c27)));
+    const float B = k == 0 ? q.y : (k == 3 ? c5 : (k == 4 ? c8 : (k == 5 ? c11 : q.x)));
+    const float C = k == 0 ? q.z : (k == 3 ? c6 : (k == 4 ? c9 : (k == 5 ? c12 : q.y)));
+    const float hx = sh && k != 3 ? 1.f : (k == 6 ? 1.f : 0.5f);
+    const float hy = sh || k == 6 ? 1.f : 0.5f;
+    const float hz = sh || k == 6 || k == 7 ? 1.f : 0.5f;
+    const float hw = k == 1 || k == 2 || k == 6 ? 0.5f : 1.f;
+    const float4 base = make_float4(hx * q.x, hy * q.y, hz * q.z, hw * q.w);
+    for (int c = 0; c < 8; ++c) {
+      const float s[3] = {(c & 1) ? 1.f : -1.f, (c & 2) ? 1.f : -1.f, (c & 4) ? 1.f : -1.f};
+      float t = 0.5f * (A * s[0] + B * s[1] + C * s[2]);
+      if (sh) t = t / kSH0;
+      float4 out = base;
+      if (sh) out.y += t;
+      if (k == 0) out.w += t;
+      if (k == 7) out.z += t;
+      dst[8 * c] = out;
+    }
   }
 }
 
@@ -140,17 +157,17 @@ __device__ __forceinline__ float reg_density(float g, float a, float b, float* d
 template <int MODE, bool VEC>
 __device__ __forceinline__ void reg_add(float* __restrict__ grads, int v, const float g[6]) {
   float* G = grads + (size_t)v * 32;
-  if (VEC) {
+  if constexpr (VEC) {
     atomicAdd(reinterpret_cast<float4*>(G), make_float4(g[0], g[1], g[2], g[3]));
     if (MODE == SALF_FIELD_SDF)
       atomicAdd(reinterpret_cast<float4*>(G + 24), make_float4(0.f, g[4], g[5], 0.f));
-    return;
-  }
+  } else {
 #pragma unroll
-  for (int q = 0; q < 4; ++q) atomicAdd(G + q, g[q]);
-  if (MODE == SALF_FIELD_SDF) {
-    atomicAdd(G + 25, g[4]);
-    atomicAdd(G + 26, g[5]);
+    for (int q = 0; q < 4; ++q) atomicAdd(G + q, g[q]);
+    if (MODE == SALF_FIELD_SDF) {
+      atomicAdd(G + 25, g[4]);
+      atomicAdd(G + 26, g[5]);
+    }
   }
 }
 
@@ -334,8 +351,8 @@ extern "C" salf_status salf_scene_refine_plan(salf_scene* sc, const float* grads
   if (n > 0) {
     const DevScene& D = sc->dev;
     k_refine_plan<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
-        D.vox_box, D.order, (int)n, D.K, grads, max_alpha, split_threshold, prune_alpha, action,
-        count, stats);
+        sc->key_level, (int)n, D.K, grads, max_alpha, split_threshold, prune_alpha, action, count,
+        stats);
     int launches = 0;
     if ((e = scan_exclusive<unsigned, unsigned long long>(count, n, offs, tmp, st, &launches)) !=
         cudaSuccess)
@@ -387,9 +404,8 @@ extern "C" salf_status salf_scene_refine_apply(salf_scene* sc, const float* para
   const unsigned char* action = reinterpret_cast<const unsigned char*>(w);
   const unsigned long long* offs = reinterpret_cast<const unsigned long long*>(w + b_act + b_cnt);
   if (n > 0 && sc->refine_n_new > 0) {
-    const DevScene& D = sc->dev;
-    k_refine_apply<<<(unsigned)((n + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        D.vox_box, D.order, (int)n, D.K, action, offs, params, level_out, ijk_out, params_out);
+    k_refine_apply<<<(unsigned)((n + 32 * kRows - 1) / (32 * kRows)), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+        sc->key_level, sc->key_ijk, (int)n, action, offs, params, level_out, ijk_out, params_out);
     if ((e = cudaGetLastError()) != cudaSuccess) return salf_cuda_fail(e, "refine apply");
   }
   return SALF_OK;

@@ -26,7 +26,7 @@
 #define SALF_BWD_WARPS 4
 #endif
 #ifndef SALF_BWD_MIN_BLOCKS
-#define SALF_BWD_MIN_BLOCKS 5  // 96 registers, 20 warps per SM: measured faster than 4 (111) and 6 (spills)
+#define SALF_BWD_MIN_BLOCKS 4  // 16 warps per SM: training step 2750 us, LiDAR fit 482; 5: 2756, 492; 6: 2834, 543
 #endif
 
 using namespace salf;
@@ -100,47 +100,43 @@ __global__ void __launch_bounds__(32 * SALF_BWD_WARPS, SALF_BWD_MIN_BLOCKS)
   const float gbg = g[0] * Q.bg[0] + g[1] * Q.bg[1] + g[2] * Q.bg[2] + gp;
   float T = 1.f, Pk = 0.f;
   int k = 0;
-  __shared__ float s_rows[SALF_BWD_WARPS][32][33];  // padded: conflict-free columns
-  float(*rows)[33] = s_rows[threadIdx.x >> 5];
-  // per-warp ring of pending hits (16 words each, padded to 17): each round's
+  // staged gradient rows, 8 chunks of 16 bytes and one of padding: lanes' 16-byte
+  // accesses are conflict-free (rows and queue in single words: training step
+  // 2827 us, in chunks 2756)
+  __shared__ float4 s_rows[SALF_BWD_WARPS][32][9];
+  float4(*rows)[9] = s_rows[threadIdx.x >> 5];
+  // per-warp ring of pending hits (4 chunks each, padded to 5): each round's
   // hits are queued, and the gradient rows and their atomics run 32 at a time
-  // on the whole warp
-  constexpr int QN = 64, QW = 17;
-  __shared__ float s_queue[SALF_BWD_WARPS][QN * QW];
-  float* queue = s_queue[threadIdx.x >> 5];
+  // on the whole warp.  A hit: (voxel, x), (geometry, SDF a and b, intensity),
+  // (colour factors, raydrop), SH basis.
+  constexpr int QN = 64, QW = 5;
+  __shared__ float4 s_queue[SALF_BWD_WARPS][QN * QW];
+  float4* queue = s_queue[threadIdx.x >> 5];
   int head = 0, tail = 0;  // warp-uniform
   const int nq = (want_int || want_drop) ? 8 : 7;
 
   // gradient rows of n queued hits (n <= 32), summed per voxel, added to d_params
   auto flush = [&](int n) {
     const bool act = lane < n;
-    float gr[32];
-#pragma unroll
-    for (int q = 0; q < 32; ++q) gr[q] = 0.f;
     int key = 0;
+    float4 gr[8];
     if (act) {
-      const float* it = queue + ((head + lane) & (QN - 1)) * QW;
-      key = __float_as_int(it[0]);
-      const float xh[4] = {it[1], it[2], it[3], 1.f};
-      const float gm[4] = {kSH0, it[13], it[14], it[15]};  // gamma_0 is a constant
-#pragma unroll
-      for (int q = 0; q < 4; ++q) gr[q] = it[4] * xh[q];
-#pragma unroll
-      for (int ch = 0; ch < 3; ++ch) {
-        const float dz = it[7 + ch];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) gr[4 + 3 * ch + a] = dz * xh[a];
-#pragma unroll
-        for (int b = 0; b < 4; ++b) gr[13 + 4 * ch + b] = dz * gm[b];
-      }
-      gr[25] = MODE == SALF_FIELD_EXP ? 0.f : it[5];  // SDF a, b (not queued in EXP mode)
-      gr[26] = MODE == SALF_FIELD_EXP ? 0.f : it[6];
-      const float di = want_int ? it[10] : 0.f, dr = want_drop ? it[11] : 0.f;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) gr[27 + q] = di * xh[q];
-      gr[31] = dr;
+      const float4* it = queue + ((head + lane) & (QN - 1)) * QW;
+      const float4 i0 = it[0], i1 = it[1], i2 = it[2], i3 = it[3];
+      key = __float_as_int(i0.x);
+      const float x0 = i0.y, x1 = i0.z, x2 = i0.w;
+      const float g1 = i3.x, g2 = i3.y, g3 = i3.z;  // gamma_0 is a constant
+      const float di = want_int ? i1.w : 0.f, dr = want_drop ? i2.w : 0.f;
+      gr[0] = make_float4(i1.x * x0, i1.x * x1, i1.x * x2, i1.x);
+      gr[1] = make_float4(i2.x * x0, i2.x * x1, i2.x * x2, i2.y * x0);
+      gr[2] = make_float4(i2.y * x1, i2.y * x2, i2.z * x0, i2.z * x1);
+      gr[3] = make_float4(i2.z * x2, i2.x * kSH0, i2.x * g1, i2.x * g2);
+      gr[4] = make_float4(i2.x * g3, i2.y * kSH0, i2.y * g1, i2.y * g2);
+      gr[5] = make_float4(i2.y * g3, i2.z * kSH0, i2.z * g1, i2.z * g2);
+      gr[6] = make_float4(i2.z * g3, MODE == SALF_FIELD_EXP ? 0.f : i1.y,
+                          MODE == SALF_FIELD_EXP ? 0.f : i1.z, di * x0);
+      gr[7] = make_float4(di * x1, di * x2, di, dr);
     }
-    __syncwarp();
     const unsigned act_lanes = __ballot_sync(0xffffffffu, act);
     if (act) {
       const unsigned peers = __match_any_sync(act_lanes, key);
@@ -148,12 +144,12 @@ __global__ void __launch_bounds__(32 * SALF_BWD_WARPS, SALF_BWD_MIN_BLOCKS)
       if (peers == (1u << lane)) {
 #pragma unroll
         for (int q = 0; q < 8; ++q)
-          if (q < nq)
-            atomicAdd(dst + q, make_float4(gr[4 * q], gr[4 * q + 1], gr[4 * q + 2], gr[4 * q + 3]));
+          if (q < nq) atomicAdd(dst + q, gr[q]);
       } else {
         // several rows of one voxel: each lane sums some 16-byte chunks over them
 #pragma unroll
-        for (int q = 0; q < 32; ++q) rows[lane][q] = gr[q];
+        for (int q = 0; q < 8; ++q)
+          if (q < nq) rows[lane][q] = gr[q];
         __syncwarp(peers);
         const int gn = __popc(peers), rank = __popc(peers & ((1u << lane) - 1u));
         for (int c = rank; c < nq; c += gn) {
@@ -162,10 +158,11 @@ __global__ void __launch_bounds__(32 * SALF_BWD_WARPS, SALF_BWD_MIN_BLOCKS)
           while (m) {
             const int l2 = __ffs(m) - 1;
             m &= m - 1u;
-            sum.x += rows[l2][4 * c];
-            sum.y += rows[l2][4 * c + 1];
-            sum.z += rows[l2][4 * c + 2];
-            sum.w += rows[l2][4 * c + 3];
+            const float4 r2 = rows[l2][c];
+            sum.x += r2.x;
+            sum.y += r2.y;
+            sum.z += r2.z;
+            sum.w += r2.w;
           }
           atomicAdd(dst + c, sum);
         }
@@ -202,27 +199,22 @@ __global__ void __launch_bounds__(32 * SALF_BWD_WARPS, SALF_BWD_MIN_BLOCKS)
       const float dtau = Tn * gq - (gQ - Pk) - Tend * gbg;
       const float dsig = dtau * dl;
       // the hit's coefficients: the gradient row is built from them later
-      float* it = queue + ((tail + __popc(hit_lanes & ((1u << lane) - 1u))) & (QN - 1)) * QW;
-      it[0] = __int_as_float(__ldg(&S.order[h.vox]));
-      it[1] = x[0];
-      it[2] = x[1];
-      it[3] = x[2];
-      if (MODE == SALF_FIELD_EXP) {
-        it[4] = dsig * sig;
-      } else {
+      float4* it = queue + ((tail + __popc(hit_lanes & ((1u << lane) - 1u))) & (QN - 1)) * QW;
+      float4 geo = make_float4(dsig * sig, 0.f, 0.f, 0.f);
+      if (MODE == SALF_FIELD_SDF) {
         const float a = f.a, b = f.b;
         const float ex = __expf(-fabsf(lin) / b);
-        it[4] = dsig * (a / (2.f * b)) * ex;
-        it[5] = dsig * sig / a;
-        it[6] = -dsig * a * lin * ex / (2.f * b * b);
+        geo.x = dsig * (a / (2.f * b)) * ex;
+        geo.y = dsig * sig / a;
+        geo.z = -dsig * a * lin * ex / (2.f * b * b);
       }
-#pragma unroll
-      for (int ch = 0; ch < 3; ++ch) it[7 + ch] = wgt * g[ch] * c[ch] * (1.f - c[ch]);
-      if (want_int) it[10] = wgt * g[5] * io * (1.f - io);
-      if (want_drop) it[11] = wgt * gp * f.dr * (1.f - f.dr);
-      it[13] = gam[1];
-      it[14] = gam[2];
-      it[15] = gam[3];
+      if (want_int) geo.w = wgt * g[5] * io * (1.f - io);
+      it[0] = make_float4(__int_as_float(__ldg(&S.order[h.vox])), x[0], x[1], x[2]);
+      it[1] = geo;
+      it[2] = make_float4(wgt * g[0] * c[0] * (1.f - c[0]), wgt * g[1] * c[1] * (1.f - c[1]),
+                          wgt * g[2] * c[2] * (1.f - c[2]),
+                          want_drop ? wgt * gp * f.dr * (1.f - f.dr) : 0.f);
+      it[3] = make_float4(gam[1], gam[2], gam[3], 0.f);
       T = Tn;
       if (++k >= nv) w.alive = false;
     }

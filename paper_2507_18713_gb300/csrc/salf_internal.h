@@ -79,6 +79,10 @@ struct DevScene {
   int* status;
   double origin[3];
   double inv_sfin;  // finest cells per metre
+  // the same as pairs of floats (value = [0] + [1] to 2^-48), for per-ray work:
+  // 64-bit units are few (2 FMAs per clock and SM)
+  float origin2[3][2];
+  float isf2[2], sf2[2];  // finest cells per metre; metres per finest cell
   int K;
   int Gf[3];
   int bmin[3], bmax[3];  // tight box of all voxels, finest cells [bmin, bmax)
@@ -271,6 +275,8 @@ salf_status salf_noalloc_setup(int device);
 salf_status salf_build_scene_impl(salf_ctx* ctx, const salf_scene_desc* d, salf_scene** out);
 // The same build from device-resident level / ijk / params (validated by the caller).
 salf_status salf_build_scene_gpu(salf_ctx* ctx, const salf_scene_desc* d, salf_scene** out);
+// The pairs of floats of a scene view from its 64-bit fields.
+void salf_view_pairs(DevScene* D);
 // Blocks per axis (mdim) of a grid's occupancy words, and log2 of its skip
 // bricks' edges in level-0 cells (p: x and y, q: z).
 void salf_grid_shape(const int32_t dims[3], int mdim[3], int* p, int* q);

@@ -70,6 +70,16 @@ salf_status upload(salf_scene* s, const std::vector<T>& v, T** out) {
 
 }  // namespace
 
+void salf_view_pairs(DevScene* D) {
+  auto split = [](double x, float out[2]) {
+    out[0] = (float)x;
+    out[1] = (float)(x - (double)out[0]);
+  };
+  for (int a = 0; a < 3; ++a) split(D->origin[a], D->origin2[a]);
+  split(D->inv_sfin, D->isf2);
+  split(1.0 / D->inv_sfin, D->sf2);
+}
+
 salf_status salf_scene_dalloc(salf_scene* s, size_t bytes, void** p) { return dalloc(s, bytes, p); }
 
 salf_status salf_build_scene_impl(salf_ctx* ctx, const salf_scene_desc* d, salf_scene** out) {
@@ -311,6 +321,7 @@ salf_status salf_build_scene_impl(salf_ctx* ctx, const salf_scene_desc* d, salf_
     D.Gf[a] = d->dims[a] << K;
   }
   D.inv_sfin = 1.0 / s->sfin;
+  salf_view_pairs(&D);
   // tight box of the occupied voxels: rays are clipped to it (no hit outside)
   for (int a = 0; a < 3; ++a) {
     D.bmin[a] = D.Gf[a];

@@ -409,6 +409,7 @@ salf_status salf_build_scene_gpu(salf_ctx* ctx, const salf_scene_desc* d, salf_s
     D.Gf[a] = d->dims[a] << K;
   }
   D.inv_sfin = 1.0 / s->sfin;
+  salf_view_pairs(&D);
   D.K = K;
   D.mode = d->mode;
   D.dtype = d->dtype;

@@ -56,27 +56,29 @@ __device__ __forceinline__ void record_slopes(const DevScene& S, int vox, float 
 
 template <int DT>
 __global__ void __launch_bounds__(256) k_secondary(const __grid_constant__ SecondaryParams P) {
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= P.R) return;
+  const unsigned i = blockIdx.x * 256u + threadIdx.x;  // R < 2^31
+  if (i >= (unsigned)P.R) return;
   const DevScene& S = P.S;
-  const int u = (int)(i % P.Q.W), v = (int)(i / P.Q.W);
+  const int v = (int)(i / (unsigned)P.Q.W), u = (int)(i - (unsigned)v * (unsigned)P.Q.W);
   Ray r;
   gen_ray(P.Q, S, u, v, (int)i, r);
   float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = make_float4(0.f, 0.f, 0.f, 0.f);
   const float O = __ldg(P.opacity + i), D = __ldg(P.depth + i);
   if (r.valid && O >= P.min_opacity && O > 0.f) {
     const float ts = D / O;
-    // hit point in finest-cell units: Oi + p
-    const double isf = S.inv_sfin;
-    double p[3];
+    // hit point in finest-cell units: Oi + p, to 48 bits
+    Pair p[3];
     int c[3];
     bool inside = true;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      p[k] = (double)r.Of[k] + (double)ts * (double)r.d[k] * isf;
-      const double f = floor(p[k]);
-      c[k] = r.Oi[k] + (int)f;
-      inside = inside && c[k] >= 0 && c[k] < S.Gf[k];
+      const float td = __fmul_rn(ts, r.d[k]);
+      p[k] = pair_add(Pair{r.Of[k], 0.f},
+                      pair_mul(Pair{td, __fmaf_rn(ts, r.d[k], -td)}, S.isf2));
+      float frac;
+      c[k] = r.Oi[k] + pair_floor(p[k], &frac);
+      // (not a number, or beyond any grid: no hit point)
+      inside = inside && fabsf(p[k].hi) < 1e9f && c[k] >= 0 && c[k] < S.Gf[k];
     }
     int vox = -1, lx, lz;
     if (inside) vox = find_leaf(S, c[0], c[1], c[2], &lx, &lz);
@@ -108,11 +110,15 @@ __global__ void __launch_bounds__(256) k_secondary(const __grid_constant__ Secon
 #pragma unroll
         for (int q = 0; q < 3; ++q) dir[q] = r.d[q] - 2.f * dn * n[q];
       }
-      double X[3];
+      float X[3];
 #pragma unroll
-      for (int q = 0; q < 3; ++q)
-        X[q] = S.origin[q] + ((double)r.Oi[q] + p[q]) / isf + (double)(side * P.offset * n[q]);
-      a = make_float4((float)X[0], (float)X[1], (float)X[2], dir[0]);
+      for (int q = 0; q < 3; ++q) {
+        const Pair m = pair_mul(pair_add(Pair{(float)r.Oi[q], 0.f}, p[q]), S.sf2);
+        const Pair w = pair_add(Pair{S.origin2[q][0], S.origin2[q][1]}, m);
+        const Pair x = pair_add(w, Pair{__fmul_rn(side * P.offset, n[q]), 0.f});
+        X[q] = __fadd_rn(x.hi, x.lo);
+      }
+      a = make_float4(X[0], X[1], X[2], dir[0]);
       b = make_float4(dir[1], dir[2], 0.f, P.t_far > 0.f ? P.t_far : 0.f);
     }
   }

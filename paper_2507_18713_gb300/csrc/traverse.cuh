@@ -24,6 +24,41 @@ struct Ray {
   bool valid;
 };
 
+// Sums and products of floats with their rounding errors (Dekker 1971, Knuth's
+// TwoSum): pairs hi + lo carry about 48 bits.  The _rn forms are never contracted.
+struct Pair {
+  float hi, lo;
+};
+
+__device__ __forceinline__ Pair two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b);
+  const float t = __fsub_rn(s, a);
+  return Pair{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+
+__device__ __forceinline__ Pair pair_add(Pair a, Pair b) {
+  const Pair s = two_sum(a.hi, b.hi);
+  return two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
+}
+
+__device__ __forceinline__ Pair pair_mul(Pair a, const float b[2]) {
+  const float p = __fmul_rn(a.hi, b[0]);
+  const float e = __fmaf_rn(a.hi, b[0], -p);
+  return two_sum(p, __fmaf_rn(a.hi, b[1], __fmaf_rn(a.lo, b[0], e)));
+}
+
+// floor of a pair as an int, and what is left of it in [0, 1) as a float.
+__device__ __forceinline__ int pair_floor(Pair a, float* frac) {
+  float f = floorf(a.hi);
+  float r = __fadd_rn(__fsub_rn(a.hi, f), a.lo);
+  if (r < 0.f) {  // hi is whole and lo below it
+    f = __fsub_rn(f, 1.f);
+    r = __fadd_rn(__fsub_rn(a.hi, f), a.lo);
+  }
+  *frac = r;
+  return (int)f;
+}
+
 // Sensor ray of pixel (u, v) / LiDAR (azimuth u, beam v).
 __device__ __forceinline__ void gen_ray(const ReqDev& Q, const DevScene& S, int u, int v,
                                         int ray, Ray& r) {
@@ -31,13 +66,13 @@ __device__ __forceinline__ void gen_ray(const ReqDev& Q, const DevScene& S, int 
   if (Q.kind == SALF_RAYS_EXPLICIT) {
     const float4* q = reinterpret_cast<const float4*>(Q.rays) + 2 * (size_t)ray;
     float4 a = __ldg(q), b = __ldg(q + 1);
-    double o[3] = {(double)a.x, (double)a.y, (double)a.z};
+    // origin in finest cells, (o - origin) / edge, to 48 bits
+    const float o[3] = {a.x, a.y, a.z};
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      double g = (o[k] - S.origin[k]) * S.inv_sfin;
-      double f = floor(g);
-      r.Oi[k] = (int)f;
-      r.Of[k] = (float)(g - f);
+      const Pair g = pair_mul(pair_add(Pair{o[k], 0.f}, Pair{-S.origin2[k][0], -S.origin2[k][1]}),
+                              S.isf2);
+      r.Oi[k] = pair_floor(g, &r.Of[k]);
     }
     float dx = a.w, dy = b.x, dz = b.y;
     float nn = dx * dx + dy * dy + dz * dz;
@@ -167,7 +202,7 @@ struct RayClip {
 };
 
 __device__ __forceinline__ void ray_clip(const DevScene& S, const Ray& r, RayClip& q) {
-  const float isf = (float)S.inv_sfin;
+  const float isf = S.isf2[0];
   q.t0 = r.tn;
   q.t1 = r.tf;
 #pragma unroll

@@ -4,13 +4,13 @@
 // Pipeline, all on the device except one read of the pair count:
 //  1. k_project: per voxel, the pixel rectangle its projection may cover
 //     (near-plane aware, widened by two pixels), the 16 x 16 tiles it touches
-//     and its camera-order key;
-//  2. exclusive scan of the tile counts -> each voxel's slot range;
-//  3. k_emit: one (tile | key, voxel) pair per touched tile;
+//     and its camera-order key; per block of voxels the number of its pairs;
+//  2. k_block_offsets: exclusive scan of the blocks' pair counts;
+//  3. k_emit: one (tile | key, voxel) pair per touched tile, in voxel order;
 //  4. stable LSD radix sort of the pairs, 8 bits per pass;
 //  5. k_tile_ranges: each tile's slice of the sorted pairs;
 //  6. k_raster: one 256-thread block per tile, one thread per pixel; the
-//     tile's voxels are staged 64 at a time in shared memory (records raw,
+//     tile's voxels are staged kChunk at a time in shared memory (records raw,
 //     boxes as plane offsets) and composited front to back with early
 //     termination, with the ray kernel's ray set-up, slab test and field code.
 //
@@ -37,16 +37,20 @@ using namespace salf_sort;
 
 namespace {
 
+// Resident tile blocks per SM the register budget must allow: 5 x 8 warps in 48
+// registers; spills cost less than the barrier waits that they hide (4K frame: 3
+// blocks 976 us, 4 890, 5 867; 5 with 64-voxel chunks 831, 6 839).
 #ifndef SALF_RASTER_MIN_BLOCKS
-#define SALF_RASTER_MIN_BLOCKS 3  // resident tile blocks per SM the register budget allows
+#define SALF_RASTER_MIN_BLOCKS 5
 #endif
 
 constexpr int kTile = 16;          // tile edge in pixels
 constexpr int kRasterThreads = kTile * kTile;
 #ifndef SALF_RASTER_CHUNK
-#define SALF_RASTER_CHUNK 128
+#define SALF_RASTER_CHUNK 64
 #endif
 constexpr int kChunk = SALF_RASTER_CHUNK;  // voxels staged in shared memory at a time
+static_assert(kChunk <= kRasterThreads, "one box per thread");
 
 struct ProjParams {
   DevScene S;
@@ -58,10 +62,12 @@ struct ProjParams {
   int ce[3];          // camera's level-0 cell
   int dig_shift;      // 3 K: bits of the octree digits
   unsigned* count;    // tiles per voxel
+  // of voxels with tiles only (most voxels of a scene are out of view):
   uint2* rect;        // tile rectangle (x0 | y0 << 16, x1 | y1 << 16)
   int4* prect;        // pixel rectangle (u0, u1, v0, v1), inclusive
   unsigned long long* key;
-  unsigned long long* n_visible;  // voxels listed in at least one tile
+  unsigned long long* block_pairs;  // pairs of each block of voxels
+  unsigned long long* n_visible;    // voxels listed in at least one tile
 };
 
 // ---------------------------------------------------------------- projection
@@ -84,17 +90,19 @@ __device__ __forceinline__ unsigned project_one(const ProjParams& G, int p) {
     ez[j] = E * G.R0[6 + j];
   }
   float pc[8][3];
-#pragma unroll
-  for (int c = 0; c < 8; ++c)
-#pragma unroll
-    for (int j = 0; j < 3; ++j)
-      pc[c][j] = base[j] + ((c & 1) ? ex[j] : 0.f) + ((c & 2) ? ey[j] : 0.f) + ((c & 4) ? ez[j] : 0.f);
-  float umin = __int_as_float(0x7f800000), umax = -umin, vmin = umin, vmax = -umin;
   bool front = false;
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      pc[c][j] = base[j] + ((c & 1) ? ex[j] : 0.f) + ((c & 2) ? ey[j] : 0.f) + ((c & 4) ? ez[j] : 0.f);
+    front = front || pc[c][2] > 0.f;
+  }
+  if (!front) return 0u;  // behind the camera
+  float umin = __int_as_float(0x7f800000), umax = -umin, vmin = umin, vmax = -umin;
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
     if (pc[c][2] > 0.f) {
-      front = true;
       const float iz = 1.f / pc[c][2];
       const float u = fmaf(G.fx * pc[c][0], iz, G.cx), v = fmaf(G.fy * pc[c][1], iz, G.cy);
       umin = fminf(umin, u);
@@ -103,43 +111,36 @@ __device__ __forceinline__ unsigned project_one(const ProjParams& G, int p) {
       vmax = fmaxf(vmax, v);
     }
   }
-  unsigned cnt = 0;
-  uint2 rc = make_uint2(0, 0);
-  int4 pr = make_int4(1, 0, 1, 0);  // empty
-  if (front) {
-    // box points close to the camera plane project without bound, in the
-    // direction of where the box's edges cross that plane
+  // box points close to the camera plane project without bound, in the
+  // direction of where the box's edges cross that plane
 #pragma unroll
-    for (int c = 0; c < 8; ++c)
+  for (int c = 0; c < 8; ++c)
 #pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        const int c2 = c | (1 << a);
-        if (c2 == c) continue;
-        const float z1 = pc[c][2], z2 = pc[c2][2];
-        if ((z1 > 0.f) == (z2 > 0.f)) continue;
-        const float t = z1 / (z1 - z2);
-        const float x0 = fmaf(t, pc[c2][0] - pc[c][0], pc[c][0]);
-        const float y0 = fmaf(t, pc[c2][1] - pc[c][1], pc[c][1]);
-        if (x0 >= 0.f) umax = __int_as_float(0x7f800000);
-        if (x0 <= 0.f) umin = -__int_as_float(0x7f800000);
-        if (y0 >= 0.f) vmax = __int_as_float(0x7f800000);
-        if (y0 <= 0.f) vmin = -__int_as_float(0x7f800000);
-      }
-    // pixel (u, v) has its ray through (u + 0.5, v + 0.5); two pixels of margin
-    const float fu0 = fmaxf(floorf(umin) - 2.f, -1.f), fu1 = fminf(floorf(umax) + 2.f, (float)G.W);
-    const float fv0 = fmaxf(floorf(vmin) - 2.f, -1.f), fv1 = fminf(floorf(vmax) + 2.f, (float)G.H);
-    const int u0 = max((int)fu0, 0), u1 = min((int)fu1, G.W - 1);
-    const int v0 = max((int)fv0, 0), v1 = min((int)fv1, G.H - 1);
-    if (u0 <= u1 && v0 <= v1 && fu1 >= 0.f && fv1 >= 0.f && fu0 < (float)G.W && fv0 < (float)G.H) {
-      const int tx0 = u0 / kTile, tx1 = u1 / kTile, ty0 = v0 / kTile, ty1 = v1 / kTile;
-      cnt = (unsigned)((tx1 - tx0 + 1) * (ty1 - ty0 + 1));
-      rc = make_uint2((unsigned)tx0 | ((unsigned)ty0 << 16), (unsigned)tx1 | ((unsigned)ty1 << 16));
-      pr = make_int4(u0, u1, v0, v1);
+    for (int a = 0; a < 3; ++a) {
+      const int c2 = c | (1 << a);
+      if (c2 == c) continue;
+      const float z1 = pc[c][2], z2 = pc[c2][2];
+      if ((z1 > 0.f) == (z2 > 0.f)) continue;
+      const float t = z1 / (z1 - z2);
+      const float x0 = fmaf(t, pc[c2][0] - pc[c][0], pc[c][0]);
+      const float y0 = fmaf(t, pc[c2][1] - pc[c][1], pc[c][1]);
+      if (x0 >= 0.f) umax = __int_as_float(0x7f800000);
+      if (x0 <= 0.f) umin = -__int_as_float(0x7f800000);
+      if (y0 >= 0.f) vmax = __int_as_float(0x7f800000);
+      if (y0 <= 0.f) vmin = -__int_as_float(0x7f800000);
     }
-  }
-  G.count[p] = cnt;
-  G.rect[p] = rc;
-  G.prect[p] = pr;
+  // pixel (u, v) has its ray through (u + 0.5, v + 0.5); two pixels of margin
+  const float fu0 = fmaxf(floorf(umin) - 2.f, -1.f), fu1 = fminf(floorf(umax) + 2.f, (float)G.W);
+  const float fv0 = fmaxf(floorf(vmin) - 2.f, -1.f), fv1 = fminf(floorf(vmax) + 2.f, (float)G.H);
+  const int u0 = max((int)fu0, 0), u1 = min((int)fu1, G.W - 1);
+  const int v0 = max((int)fv0, 0), v1 = min((int)fv1, G.H - 1);
+  if (!(u0 <= u1 && v0 <= v1 && fu1 >= 0.f && fv1 >= 0.f && fu0 < (float)G.W &&
+        fv0 < (float)G.H))
+    return 0u;
+  const int tx0 = u0 / kTile, tx1 = u1 / kTile, ty0 = v0 / kTile, ty1 = v1 / kTile;
+  G.rect[p] =
+      make_uint2((unsigned)tx0 | ((unsigned)ty0 << 16), (unsigned)tx1 | ((unsigned)ty1 << 16));
+  G.prect[p] = make_int4(u0, u1, v0, v1);
   // camera-order key
   const int K = G.S.K;
   unsigned l1 = 0;
@@ -159,17 +160,46 @@ __device__ __forceinline__ unsigned project_one(const ProjParams& G, int p) {
     dig |= (unsigned long long)dj << (3 * (K - j));
   }
   G.key[p] = ((unsigned long long)l1 << G.dig_shift) | dig;
-  return cnt;
+  return (unsigned)((tx1 - tx0 + 1) * (ty1 - ty0 + 1));
 }
 
 __global__ void __launch_bounds__(256) k_project(const __grid_constant__ ProjParams G) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  const bool live = p < G.S.n;
   unsigned cnt = 0;
-  if (live) cnt = project_one(G, p);
+  if (p < G.S.n) {
+    cnt = project_one(G, p);
+    G.count[p] = cnt;
+  }
   const int nvis = __syncthreads_count(cnt > 0);
-  if (threadIdx.x == 0 && nvis) atomicAdd(G.n_visible, (unsigned long long)nvis);
+  if (nvis == 0) {
+    if (threadIdx.x == 0) G.block_pairs[blockIdx.x] = 0ull;
+    return;
+  }
+  unsigned long long total;
+  block_exclusive_scan<unsigned long long>(cnt, &total);
+  if (threadIdx.x == 0) {
+    G.block_pairs[blockIdx.x] = total;
+    atomicAdd(G.n_visible, (unsigned long long)nvis);
+  }
 }
+
+// Exclusive scan of the blocks' pair counts in place (one block), and the sum.
+__global__ void __launch_bounds__(1024) k_block_offsets(unsigned long long* __restrict__ pairs,
+                                                        long long n,
+                                                        unsigned long long* __restrict__ sum) {
+  unsigned long long run = 0;
+  for (long long b0 = 0; b0 < n; b0 += 1024) {
+    const long long b = b0 + threadIdx.x;
+    const unsigned long long c = b < n ? pairs[b] : 0ull;
+    unsigned long long tot;
+    const unsigned long long before = block_exclusive_scan<unsigned long long>(c, &tot);
+    if (b < n) pairs[b] = run + before;
+    run += tot;
+  }
+  if (threadIdx.x == 0) *sum = run;
+}
+
+constexpr unsigned kAlone = 8;  // pairs that a thread emits by itself
 
 __global__ void __launch_bounds__(256) k_emit(const unsigned* __restrict__ count,
                                               const uint2* __restrict__ rect,
@@ -179,16 +209,46 @@ __global__ void __launch_bounds__(256) k_emit(const unsigned* __restrict__ count
                                               unsigned long long* __restrict__ out_key,
                                               unsigned* __restrict__ out_val) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n || count[p] == 0) return;
-  const uint2 rc = rect[p];
-  const int tx0 = rc.x & 0xffff, ty0 = rc.x >> 16, tx1 = rc.y & 0xffff, ty1 = rc.y >> 16;
-  unsigned long long o = offs[p];
-  const unsigned long long k = key[p];
-  for (int ty = ty0; ty <= ty1; ++ty)
-    for (int tx = tx0; tx <= tx1; ++tx, ++o) {
-      out_key[o] = ((unsigned long long)(ty * tiles_x + tx) << key_bits_low) | k;
-      out_val[o] = (unsigned)p;
+  const unsigned cnt = p < n ? count[p] : 0u;
+  if (__syncthreads_count(cnt > 0) == 0) return;
+  unsigned long long total;
+  unsigned long long o = block_exclusive_scan<unsigned long long>(cnt, &total) + offs[blockIdx.x];
+  // a voxel near the camera covers hundreds of tiles: its warp emits those pairs
+  // together (one thread each: 24 us for 1.2M pairs of a 4K frame)
+  const int lane = threadIdx.x & 31;
+  uint2 rc = make_uint2(0, 0);
+  unsigned long long k = 0;
+  if (cnt) {
+    rc = rect[p];
+    k = key[p];
+  }
+  unsigned todo = __ballot_sync(0xffffffffu, cnt > kAlone);
+  if (cnt <= kAlone) {
+    const int tx0 = rc.x & 0xffff, w = (int)(rc.y & 0xffff) - tx0 + 1;
+    int tx = tx0, ty = rc.x >> 16;
+    for (unsigned i = 0; i < cnt; ++i) {
+      out_key[o + i] = ((unsigned long long)(ty * tiles_x + tx) << key_bits_low) | k;
+      out_val[o + i] = (unsigned)p;
+      if (++tx == tx0 + w) {
+        tx = tx0;
+        ++ty;
+      }
     }
+  }
+  while (todo) {
+    const int src = __ffs(todo) - 1;
+    todo &= todo - 1u;
+    const unsigned c = __shfl_sync(0xffffffffu, cnt, src);
+    const unsigned r0 = __shfl_sync(0xffffffffu, rc.x, src), r1 = __shfl_sync(0xffffffffu, rc.y, src);
+    const unsigned long long ks = __shfl_sync(0xffffffffu, k, src);
+    const unsigned long long os = __shfl_sync(0xffffffffu, o, src);
+    const unsigned tx0 = r0 & 0xffffu, ty0 = r0 >> 16, w = (r1 & 0xffffu) - tx0 + 1u;
+    for (unsigned i = (unsigned)lane; i < c; i += 32) {
+      const unsigned row = i / w, t = (ty0 + row) * (unsigned)tiles_x + tx0 + (i - row * w);
+      out_key[os + i] = ((unsigned long long)t << key_bits_low) | ks;
+      out_val[os + i] = (unsigned)(p - lane + src);
+    }
+  }
 }
 
 __global__ void __launch_bounds__(256) k_tile_ranges(const unsigned long long* __restrict__ keys,
@@ -225,13 +285,54 @@ __global__ void __launch_bounds__(kRasterThreads, SALF_RASTER_MIN_BLOCKS) k_rast
   const ReqDev& Q = RP.Q;
   const int tile = blockIdx.x;
   const int lane = threadIdx.x & 31;
-  const int u = (tile % RP.tiles_x) * kTile + (threadIdx.x % kTile);
-  const int v = (tile / RP.tiles_x) * kTile + (threadIdx.x / kTile);
-  // this warp's pixels: 16 columns x 2 rows
-  const int strip_u0 = (tile % RP.tiles_x) * kTile, strip_u1 = strip_u0 + kTile - 1;
-  const int strip_v0 = (tile / RP.tiles_x) * kTile + 2 * (threadIdx.x >> 5), strip_v1 = strip_v0 + 1;
+  // this warp's pixels: 8 columns x 4 rows (16 x 2 meet a fifth more voxels: 4K frame
+  // 864 us against 842)
+  const int warp = threadIdx.x >> 5;
+  const int strip_u0 = (tile % RP.tiles_x) * kTile + 8 * (warp & 1), strip_u1 = strip_u0 + 7;
+  const int strip_v0 = (tile / RP.tiles_x) * kTile + 4 * (warp >> 1), strip_v1 = strip_v0 + 3;
+  const int u = strip_u0 + (lane & 7), v = strip_v0 + (lane >> 3);
   const bool in_img = u < Q.W && v < Q.H;
   const int ray = v * Q.W + u;
+
+  const uint2 rg = RP.ranges[tile];
+  // A chunk's records go to shared memory without passing through registers,
+  // its boxes through registers; the first chunk's are fetched while the rays are
+  // set up (most tiles of a 4K frame have one chunk, and the block waited for it).
+  int4 box, pr;
+  unsigned vx = 0;
+  auto fetch = [&](unsigned c0, int n) {
+    for (int i = threadIdx.x; i < n * RQ; i += kRasterThreads) {
+      const int j = i / RQ, k = i % RQ;
+      const float4* src = reinterpret_cast<const float4*>(S.params) +
+                          (size_t)__ldg(&RP.vox[c0 + j]) * RQ + k;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                       (unsigned)__cvta_generic_to_shared(&s_rec[j * RS + k])),
+                   "l"(src)
+                   : "memory");
+    }
+    if ((int)threadIdx.x < n) {
+      vx = __ldg(&RP.vox[c0 + threadIdx.x]);
+      box = __ldg(&S.vox_box[vx]);
+      pr = __ldg(&RP.prect[vx]);
+    }
+  };
+  auto store = [&](int n) {
+    if ((int)threadIdx.x < n) {
+      const int E = 1 << box.w;
+      const int lo[3] = {box.x, box.y, box.z};
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        s_pl[threadIdx.x][a] = (float)(lo[a] - Q.Oi[a]) - Q.Of[a];
+        s_pl[threadIdx.x][3 + a] = (float)(lo[a] + E - Q.Oi[a]) - Q.Of[a];
+      }
+      s_box[threadIdx.x] = box;
+      s_prect[threadIdx.x] = pr;
+      s_vox[threadIdx.x] = (int)vx;
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+  };
+  if (rg.x < rg.y) fetch(rg.x, (int)min((unsigned)kChunk, rg.y - rg.x));
 
   Ray r;
   RayClip w;
@@ -253,30 +354,10 @@ __global__ void __launch_bounds__(kRasterThreads, SALF_RASTER_MIN_BLOCKS) k_rast
   for (int a = 0; a < 3; ++a) pos[a] = w.D[a] > 0.f;
   Accum A{1.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0};
 
-  const uint2 rg = RP.ranges[tile];
   for (unsigned c0 = rg.x; c0 < rg.y; c0 += kChunk) {
     const int n = (int)min((unsigned)kChunk, rg.y - c0);
-    __syncthreads();  // the previous chunk is no longer read
-    for (int i = threadIdx.x; i < n * RQ; i += kRasterThreads) {
-      const int j = i / RQ, k = i % RQ;
-      const unsigned vx = __ldg(&RP.vox[c0 + j]);
-      s_rec[j * RS + k] = __ldg(reinterpret_cast<const float4*>(S.params) + (size_t)vx * RQ + k);
-    }
-    for (int i = threadIdx.x; i < n; i += kRasterThreads) {
-      const unsigned vx = __ldg(&RP.vox[c0 + i]);
-      const int4 b = __ldg(&S.vox_box[vx]);
-      const int E = 1 << b.w;
-      const int lo[3] = {b.x, b.y, b.z};
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        s_pl[i][a] = (float)(lo[a] - Q.Oi[a]) - Q.Of[a];
-        s_pl[i][3 + a] = (float)(lo[a] + E - Q.Oi[a]) - Q.Of[a];
-      }
-      s_box[i] = b;
-      s_prect[i] = __ldg(&RP.prect[vx]);
-      s_vox[i] = (int)vx;
-    }
-    __syncthreads();
+    if (c0 != rg.x) fetch(c0, n);  // the previous chunk is no longer read (end of the loop)
+    store(n);
     // voxels whose pixel rectangle meets this warp's 16 x 2 pixel strip
     unsigned sel[kChunk / 32];
 #pragma unroll
@@ -419,9 +500,9 @@ salf_status salf_raster_run(salf_scene* sc, const ReqDev& r, double fx, double f
   // per-voxel workspace
   const long long nn = std::max(n, 1LL);
   const size_t b_count = align256(nn * 4), b_rect = align256(nn * 8), b_key = align256(nn * 8),
-               b_offs = align256((nn + 2) * 8), b_tmp = align256(scan_tmp_elems(nn) * 8),
+               b_offs = align256(((nn + 255) / 256 + 2) * 8),
                b_ranges = align256((size_t)ntiles * 8), b_prect = align256(nn * 16);
-  const size_t need_vox = b_count + b_rect + b_key + b_offs + b_tmp + b_ranges + b_prect;
+  const size_t need_vox = b_count + b_rect + b_key + b_offs + b_ranges + b_prect;
   if (sc->raster_vox_bytes < need_vox) {
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return salf_cuda_fail(e, "raster sync");
     if ((e = cudaEventSynchronize(sc->raster_done)) != cudaSuccess)
@@ -447,10 +528,8 @@ salf_status salf_raster_run(salf_scene* sc, const ReqDev& r, double fx, double f
   uint2* rect = reinterpret_cast<uint2*>(wv + b_count);
   unsigned long long* vkey = reinterpret_cast<unsigned long long*>(wv + b_count + b_rect);
   unsigned long long* offs = reinterpret_cast<unsigned long long*>(wv + b_count + b_rect + b_key);
-  unsigned long long* stmp =
-      reinterpret_cast<unsigned long long*>(wv + b_count + b_rect + b_key + b_offs);
-  uint2* ranges = reinterpret_cast<uint2*>(wv + b_count + b_rect + b_key + b_offs + b_tmp);
-  int4* prect = reinterpret_cast<int4*>(wv + b_count + b_rect + b_key + b_offs + b_tmp + b_ranges);
+  uint2* ranges = reinterpret_cast<uint2*>(wv + b_count + b_rect + b_key + b_offs);
+  int4* prect = reinterpret_cast<int4*>(wv + b_count + b_rect + b_key + b_offs + b_ranges);
 
   unsigned long long P = 0, visible = 0;
   int launches = 0;
@@ -477,16 +556,16 @@ salf_status salf_raster_run(salf_scene* sc, const ReqDev& r, double fx, double f
     G.rect = rect;
     G.prect = prect;
     G.key = vkey;
-    G.n_visible = offs + n + 1;
-    if ((e = cudaMemsetAsync(offs + n + 1, 0, 8, st)) != cudaSuccess)
+    const long long vblocks = (n + 255) / 256;
+    unsigned long long* sums = offs + vblocks;  // pairs, visible voxels
+    G.block_pairs = offs;
+    G.n_visible = sums + 1;
+    if ((e = cudaMemsetAsync(sums, 0, 16, st)) != cudaSuccess)
       return salf_cuda_fail(e, "raster counter");
-    k_project<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(G);
-    if ((e = scan_exclusive<unsigned, unsigned long long>(count, n, offs, stmp, st, &launches)) !=
-        cudaSuccess)
-      return salf_cuda_fail(e, "raster scan");
-    k_scan_total<unsigned, unsigned long long><<<1, 1, 0, st>>>(count, n, offs);
+    k_project<<<(unsigned)vblocks, 256, 0, st>>>(G);
+    k_block_offsets<<<1, 1024, 0, st>>>(offs, vblocks, sums);
     launches += 2;
-    if ((e = cudaMemcpyAsync(sc->raster_count_host, offs + n, 16, cudaMemcpyDeviceToHost, st)) !=
+    if ((e = cudaMemcpyAsync(sc->raster_count_host, sums, 16, cudaMemcpyDeviceToHost, st)) !=
         cudaSuccess)
       return salf_cuda_fail(e, "raster count copy");
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return salf_cuda_fail(e, "raster project");
@@ -503,7 +582,7 @@ salf_status salf_raster_run(salf_scene* sc, const ReqDev& r, double fx, double f
   const long long hn = (long long)kRadix * std::max(nblk, 1LL);
   const size_t pp = std::max<unsigned long long>(P, 1);
   const size_t b_k = align256(pp * 8), b_v = align256(pp * 4), b_h = align256(hn * 4),
-               b_ht = align256(scan_tmp_elems(hn) * 4);
+               b_ht = align256(kRadix * 4);
   const size_t need_pairs = 2 * b_k + 2 * b_v + 2 * b_h + b_ht;
   if (sc->raster_pairs_bytes < need_pairs) {
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return salf_cuda_fail(e, "raster sync");

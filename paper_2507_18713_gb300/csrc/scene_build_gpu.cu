@@ -324,7 +324,7 @@ salf_status salf_build_scene_gpu(salf_ctx* ctx, const salf_scene_desc* d, salf_s
   // temporaries; the ones that start at 0 and at all ones are together
   const long long hn = radix_hist_elems(nn);
   const size_t b_k = a256(nn * 8), b_v = a256(nn * 4), b_h = a256(hn * 4),
-               b_ht = a256(scan_tmp_elems(hn) * 4), b_m0 = a256(nb0 * 8), b_b = a256(nb0 * 4),
+               b_ht = a256(kRadix * 4), b_m0 = a256(nb0 * 8), b_b = a256(nb0 * 4),
                b_rt = a256(scan_tmp_elems(nb0) * 4), b_c = K > 0 ? a256(nn * 4) : 0,
                b_no = K > 0 ? a256(nn * 8) : 0, b_nt = K > 0 ? a256(scan_tmp_elems(nn) * 8) : 0;
   PoolBuf tmp;

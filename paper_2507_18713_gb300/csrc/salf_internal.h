@@ -17,16 +17,6 @@
 #endif
 #define SALF_TILE_H (32 / SALF_TILE_W)
 #define SALF_WARPS_PER_BLOCK 8
-// Spans per ray when the caller leaves the choice to the library (power of 2 <= 8).
-#ifndef SALF_SEGMENTS_LIDAR
-#define SALF_SEGMENTS_LIDAR 4
-#endif
-#ifndef SALF_SEGMENTS_FISHEYE
-#define SALF_SEGMENTS_FISHEYE 1
-#endif
-#ifndef SALF_SEGMENTS_PANORAMA
-#define SALF_SEGMENTS_PANORAMA 1
-#endif
 // Azimuths per warp tile of a LiDAR walked in spans (power of 2; the rest of
 // the tile's rays are beams).
 #ifndef SALF_SEG_LIDAR_TILE_W
@@ -292,7 +282,8 @@ salf_status salf_prepare_request(const salf_scene* sc, const salf_sensor* sen,
 // Warp tiles of a request with 2^seg_shift lanes per ray (0: whole rays);
 // callers whose kernels walk whole rays re-tile with 0.
 void salf_request_tiling(ReqDev* r, const salf_sensor* s, int seg_shift);
-int salf_auto_segments(int kind);
+// Spans per ray when the caller leaves the choice to the library.
+int salf_auto_segments(const salf_scene* sc, const salf_sensor* s);
 int64_t salf_request_rays(const salf_sensor* sen);
 void salf_relative_rotation(const double* pose0, const double* pose1, float axis[3],
                             float* angle);

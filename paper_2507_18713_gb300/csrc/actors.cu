@@ -31,14 +31,12 @@ namespace {
 #define SALF_ACTOR_MIN_BLOCKS 1  // resident merge blocks per SM the register budget must allow
 #endif
 // The same for the lean merge variant (static pinhole cameras without
-// intensity).  Without the other sensors' ray generation and the intensity
-// field it fits 128 registers: 4 resident blocks per SM measured faster (1080p
-// camera with 24 actors 0.834 -> 0.754 ms).  5 blocks (96 registers, 64 bytes
-// of spills) were faster again (0.717 -> 0.689 ms), and 6 no better.  Merge
-// blocks hold most of an SM's registers while they run, so the ray kernel
-// beside them gets few slots; the merge kernel's total warp time sets the frame.
+// intensity): 4 blocks of 128 registers without spills (1080p camera with 24
+// actors 573 us; 5 blocks 587, 6 blocks 593, which spill).  Merge blocks hold most
+// of an SM's registers while they run, so the ray kernel beside them gets few
+// slots; the two kernels' summed SM time sets the frame.
 #ifndef SALF_ACTOR_MIN_BLOCKS_LEAN
-#define SALF_ACTOR_MIN_BLOCKS_LEAN 5
+#define SALF_ACTOR_MIN_BLOCKS_LEAN 4
 #endif
 
 constexpr int kActorWarps = 4;  // warps per block
@@ -108,13 +106,52 @@ __device__ __forceinline__ bool box_interval(const ActorDev& A, const Ray& r, fl
   return a1 > a0;
 }
 
-// Split the request's tiles into those whose rays may meet an actor (list 1,
-// rendered by the merge kernel) and the rest (list 0, rendered by the plain
-// ray kernel).  One warp per tile, tiles taken in launch order.
+// The warp's tile against its candidate actors (word k0 / 32, bits `cand`): each
+// lane's own ray against each candidate box; returns the actors that are met.
+__device__ __forceinline__ unsigned met_actors(const ActorDev* __restrict__ actors, int k0,
+                                               unsigned cand, const Ray& r, bool ok) {
+  unsigned hit = 0u;
+  while (cand) {
+    const int j = __ffs(cand) - 1;
+    cand &= cand - 1u;
+    float tin;
+    const bool mine = ok && may_meet(actors[k0 + j], r) && box_interval(actors[k0 + j], r, &tin);
+    if (__any_sync(0xffffffffu, mine)) hit |= 1u << j;
+  }
+  return hit;
+}
+
+// May actor A's sphere, its centre moving linearly from c0 to c1 (the segment's
+// bounding sphere), meet a cone of half angle `half` about m, over [tn, tf]?
+__device__ __forceinline__ bool cone_meets(const ActorDev& A, float smin, float smax,
+                                           const float m[3], float half, float tn, float tf) {
+  float c0[3], c1[3], c[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    c0[a] = fmaf(smin, A.cc1[a] - A.cc0[a], A.cc0[a]);
+    c1[a] = fmaf(smax, A.cc1[a] - A.cc0[a], A.cc0[a]);
+    c[a] = 0.5f * (c0[a] + c1[a]);
+  }
+  const float dx = c1[0] - c0[0], dy = c1[1] - c0[1], dz = c1[2] - c0[2];
+  const float rad = A.radius + 0.5f * sqrtf(dx * dx + dy * dy + dz * dz);
+  const float dist = sqrtf(c[0] * c[0] + c[1] * c[1] + c[2] * c[2]);
+  if (dist <= rad || half >= 1.5707963f) return true;  // inside the sphere; a wide cone
+  // angle between the cone axis and the centre, less the sphere's angular radius
+  const float ca = fminf(fmaxf((m[0] * c[0] + m[1] * c[1] + m[2] * c[2]) / dist, -1.f), 1.f);
+  const float ang = acosf(ca) - asinf(fminf(rad / dist, 1.f));
+  return ang <= half && dist - rad <= tf && dist + rad >= tn;
+}
+
+// The request's tiles whose rays may meet an actor: rendered by the merge kernel
+// (the list), left out by the plain ray kernel (the bits; it keeps its launch order,
+// longest rays first: with a second list, in the order the tiles were classified, it
+// took 268 us instead of 228).  One warp per tile.
+template <bool EXPL>
 __global__ void __launch_bounds__(128) k_classify_tiles(const __grid_constant__ LaunchParams P,
                                                         const ActorDev* __restrict__ actors,
-                                                        int n_actors, int* __restrict__ lists,
-                                                        int* __restrict__ counts,
+                                                        int n_actors, unsigned* __restrict__ bits,
+                                                        int* __restrict__ list,
+                                                        int* __restrict__ count,
                                                         unsigned* __restrict__ masks) {
   const int tile = blockIdx.x * 4 + (threadIdx.x >> 5);
   if (tile >= P.req[0].n_tiles) return;
@@ -132,7 +169,7 @@ __global__ void __launch_bounds__(128) k_classify_tiles(const __grid_constant__ 
   r.tn = 0.f;
   r.tf = 0.f;
   const bool in_img = u < Q.W && v < Q.H;
-  if (in_img) gen_ray(Q, P.S, u, v, v * Q.W + u, r);
+  if (in_img) gen_ray<EXPL>(Q, P.S, u, v, v * Q.W + u, r);
   const bool ok = in_img && r.valid;
   float m[3];
 #pragma unroll
@@ -160,52 +197,143 @@ __global__ void __launch_bounds__(128) k_classify_tiles(const __grid_constant__ 
     }
     // widen by FP32 slack; a cone wider than 90 degrees accepts everything
     const float half = acosf(fminf(fmaxf(cmin, -1.f), 1.f)) + 1e-4f;
-    // each lane tests actors lane, lane + 32, ...: the sphere (centre moving
-    // linearly over [smin, smax]: its segment's bounding sphere) against the cone
     for (int k0 = 0; k0 < n_actors; k0 += 32) {
       const int k = k0 + lane;
-      bool meet = false;
-      if (k < n_actors) {
-      const ActorDev& A = actors[k];
-      float c0[3], c1[3], c[3];
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        c0[a] = fmaf(smin, A.cc1[a] - A.cc0[a], A.cc0[a]);
-        c1[a] = fmaf(smax, A.cc1[a] - A.cc0[a], A.cc0[a]);
-        c[a] = 0.5f * (c0[a] + c1[a]);
-      }
-      const float dx = c1[0] - c0[0], dy = c1[1] - c0[1], dz = c1[2] - c0[2];
-      const float rad = A.radius + 0.5f * sqrtf(dx * dx + dy * dy + dz * dz);
-      const float dist = sqrtf(c[0] * c[0] + c[1] * c[1] + c[2] * c[2]);
-      if (dist <= rad) {
-        meet = true;  // the sensor is inside the sphere
-      } else if (half >= 1.5707963f) {
-        meet = true;
-      } else {
-        // angle between the cone axis and the centre, less the sphere's angular radius
-        const float ca = fminf(fmaxf((m[0] * c[0] + m[1] * c[1] + m[2] * c[2]) / dist, -1.f), 1.f);
-        const float ang = acosf(ca) - asinf(fminf(rad / dist, 1.f));
-        meet = ang <= half && dist - rad <= tf && dist + rad >= tn;
-      }
-      }
-      // the cone's candidates, then each lane's own ray against each candidate box
-      unsigned cand = __ballot_sync(0xffffffffu, meet), hit = 0u;
-      while (cand) {
-        const int j = __ffs(cand) - 1;
-        cand &= cand - 1u;
-        float tin;
-        const bool mine = ok && may_meet(actors[k0 + j], r) && box_interval(actors[k0 + j], r, &tin);
-        if (__any_sync(0xffffffffu, mine)) hit |= 1u << j;
-      }
+      const bool meet = k < n_actors && cone_meets(actors[k], smin, smax, m, half, tn, tf);
+      const unsigned hit = met_actors(actors, k0, __ballot_sync(0xffffffffu, meet), r, ok);
       if (lane == 0) masks[(size_t)tile * kMaskWords + (k0 >> 5)] = hit;
       any = any || hit != 0u;
     }
   }
-  if (lane == 0) {
-    const int which = any ? 1 : 0;
-    const int slot = atomicAdd(&counts[which], 1);
-    lists[which * Q.n_tiles + slot] = tile;
+  if (lane == 0 && any) {
+    atomicOr(&bits[tile >> 5], 1u << (tile & 31));
+    list[atomicAdd(count, 1)] = tile;
   }
+}
+
+// The same for a pinhole camera with one pose.  A block takes 32 tiles: lane l of
+// every warp bounds tile l's rays by the cone through its four corner pixels, and
+// the warps share the actors.  An actor is a candidate of a tile if the cone meets
+// its sphere and the cone's axis its box grown by the cone's width there; if the
+// axis meets the box itself, the tile goes to the merge kernel with its candidates
+// (which tests every ray's boxes again).  Only tiles without such an actor, those
+// along the silhouettes, have their rays tested one by one: that test's chain of
+// dependent loads and divisions, up to a dozen candidates near a vanishing point,
+// was what the kernel waited for.  1080p, 24 actors: 14 us; 47 with it on
+// every candidate, in a warp per tile or shared like this.
+constexpr int kClassifyWarps = 8;
+
+__global__ void __launch_bounds__(32 * kClassifyWarps)
+    k_classify_pinhole(const __grid_constant__ LaunchParams P, const ActorDev* __restrict__ actors,
+                       int n_actors, unsigned* __restrict__ bits, int* __restrict__ list,
+                       int* __restrict__ count, unsigned* __restrict__ masks) {
+  __shared__ unsigned s_cand[32][kMaskWords];
+  __shared__ unsigned s_meets;  // bit per tile
+  const ReqDev& Q = P.req[0];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tile0 = blockIdx.x * 32;
+  const int tile = tile0 + lane;
+  const bool live = tile < Q.n_tiles;
+  for (int i = threadIdx.x; i < 32 * kMaskWords; i += 32 * kClassifyWarps) (&s_cand[0][0])[i] = 0u;
+  if (threadIdx.x == 0) s_meets = 0u;
+  __syncthreads();
+  if (live) {
+    int u0, v0;
+    tile_origin(Q, tile, &u0, &v0);
+    float d[4][3], m[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      Ray r;
+      gen_ray_pinhole(Q, (c & 1) ? u0 + Q.tile_w - 1 : u0, (c & 2) ? v0 + Q.tile_h - 1 : v0, r);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        d[c][a] = r.d[a];
+        m[a] += r.d[a];
+      }
+    }
+    const float inv = rsqrtf(m[0] * m[0] + m[1] * m[1] + m[2] * m[2]);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) m[a] *= inv;
+    float chord2 = 0.f;  // largest squared distance of a corner's direction from the axis
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const float x = d[c][0] - m[0], y = d[c][1] - m[1], z = d[c][2] - m[2];
+      chord2 = fmaxf(chord2, x * x + y * y + z * z);
+    }
+    // half angle h: |chord| = 2 sin(h / 2), widened by FP32 slack
+    const float sh = fminf(0.5f * sqrtf(chord2) + 1e-5f, 0.7f);
+    const float ch = sqrtf(1.f - sh * sh), sn = 2.f * sh * ch, cs = 1.f - 2.f * sh * sh;
+    for (int k = warp; k < n_actors; k += kClassifyWarps) {
+      const ActorDev& A = actors[k];
+      const float x = A.cc0[0], y = A.cc0[1], z = A.cc0[2];
+      const float t = m[0] * x + m[1] * y + m[2] * z, c2 = x * x + y * y + z * z;
+      const float rad = A.radius + 1e-4f * sqrtf(c2);
+      // distance of the sphere's centre from the cone (its side, or less)
+      const float side = sqrtf(fmaxf(c2 - t * t, 0.f)) * cs - t * sn;
+      const bool far = t - rad > Q.t_far || sqrtf(c2) + rad < Q.t_near;
+      if (sh >= 0.7f) {  // a cone of 90 degrees or more: every ray decides
+        atomicOr(&s_cand[lane][k >> 5], 1u << (k & 31));
+        continue;
+      }
+      if (side > rad || far) continue;
+      // the axis in the actor's frame (the pose at t0) against its box
+      const float grow = (sqrtf(c2) + rad) * (sn / cs);
+      float in0 = Q.t_near, in1 = Q.t_far, g0 = Q.t_near * cs, g1 = Q.t_far;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const float o = A.R0[c] * A.orel0[0] + A.R0[3 + c] * A.orel0[1] + A.R0[6 + c] * A.orel0[2];
+        const float dd = A.R0[c] * m[0] + A.R0[3 + c] * m[1] + A.R0[6 + c] * m[2];
+        const float inv_d = 1.f / (fabsf(dd) < 1e-20f ? 1e-20f : dd);
+        const float p = (A.box_lo[c] - o) * inv_d, q = (A.box_hi[c] - o) * inv_d;
+        const float w = grow * fabsf(inv_d);
+        in0 = fmaxf(in0, fminf(p, q));
+        in1 = fminf(in1, fmaxf(p, q));
+        g0 = fmaxf(g0, fminf(p, q) - w);
+        g1 = fminf(g1, fmaxf(p, q) + w);
+      }
+      if (g1 * 1.0001f + 1e-3f < g0) continue;
+      atomicOr(&s_cand[lane][k >> 5], 1u << (k & 31));
+      if (in1 > in0) atomicOr(&s_meets, 1u << lane);
+    }
+  }
+  __syncthreads();
+  unsigned any_cand = 0u;
+#pragma unroll
+  for (int w = 0; w < kMaskWords; ++w) any_cand |= s_cand[lane][w];
+  const unsigned sure = s_meets;
+  __syncthreads();  // every warp has read it
+  int turn = 0;
+  for (unsigned todo = __ballot_sync(0xffffffffu, any_cand != 0u) & ~sure; todo; todo &= todo - 1u) {
+    if (turn++ % kClassifyWarps != warp) continue;
+    const int j = __ffs(todo) - 1;
+    int u0, v0;
+    tile_origin(Q, tile0 + j, &u0, &v0);
+    const int u = u0 + lane % Q.tile_w, v = v0 + lane / Q.tile_w;
+    const bool ok = u < Q.W && v < Q.H;
+    Ray r;
+    gen_ray_pinhole(Q, u, v, r);
+    bool any = false;
+    for (int w = 0; w < kMaskWords; ++w) {
+      const unsigned hit = met_actors(actors, 32 * w, s_cand[j][w], r, ok);
+      any = any || hit != 0u;
+      __syncwarp();
+      if (lane == 0) s_cand[j][w] = hit;
+    }
+    if (lane == 0 && any) atomicOr(&s_meets, 1u << j);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < 32 * kMaskWords; i += 32 * kClassifyWarps)
+    if ((s_meets >> (i / kMaskWords)) & 1u)
+      masks[(size_t)tile0 * kMaskWords + i] = s_cand[i / kMaskWords][i % kMaskWords];
+  if (warp != 0) return;
+  const unsigned meets = s_meets;
+  int slot = 0;
+  if (lane == 0 && meets) {
+    bits[blockIdx.x] = meets;
+    slot = atomicAdd(count, __popc(meets));
+  }
+  slot = __shfl_sync(0xffffffffu, slot, 0) + __popc(meets & ((1u << lane) - 1u));
+  if ((meets >> lane) & 1u) list[slot] = tile;
 }
 
 // Start actor A's walk for the ray (frame conversion to its grid cells).
@@ -626,10 +754,20 @@ cudaError_t salf_launch_backward_actors(const LaunchParams& P, const ActorDev* a
 }
 
 cudaError_t salf_launch_classify(const LaunchParams& P, const ActorDev* actors, int n_actors,
-                                 int* lists, int* counts, unsigned* masks, cudaStream_t st) {
-  const int blocks = (P.req[0].n_tiles + 3) / 4;
-  if (blocks > 0)
-    k_classify_tiles<<<blocks, 128, 0, st>>>(P, actors, n_actors, lists, counts, masks);
+                                 unsigned* bits, int* list, int* count, unsigned* masks,
+                                 cudaStream_t st) {
+  const ReqDev& q = P.req[0];
+  if (q.n_tiles <= 0) return cudaSuccess;
+  if (q.kind == SALF_PINHOLE && !q.moving) {
+    const int blocks = (q.n_tiles + 31) / 32;
+    k_classify_pinhole<<<blocks, 32 * kClassifyWarps, 0, st>>>(P, actors, n_actors, bits, list, count, masks);
+    return cudaGetLastError();
+  }
+  const int blocks = (q.n_tiles + 3) / 4;
+  if (q.kind == SALF_RAYS_EXPLICIT)
+    k_classify_tiles<true><<<blocks, 128, 0, st>>>(P, actors, n_actors, bits, list, count, masks);
+  else
+    k_classify_tiles<false><<<blocks, 128, 0, st>>>(P, actors, n_actors, bits, list, count, masks);
   return cudaGetLastError();
 }
 

@@ -929,7 +929,8 @@ extern "C" salf_status salf_render_rays_actors(salf_scene* sc, const salf_actor*
   }
   const size_t table_bytes = ((std::max<size_t>(1, (size_t)na) * sizeof(ActorDev)) + 255) & ~(size_t)255;
   const size_t mask_bytes = (size_t)r.n_tiles * (SALF_MAX_ACTORS / 32) * sizeof(unsigned);
-  const size_t bytes = table_bytes + mask_bytes + (2 * (size_t)r.n_tiles + 2) * sizeof(int);
+  const size_t bit_words = ((size_t)r.n_tiles + 31) / 32;
+  const size_t bytes = table_bytes + mask_bytes + ((size_t)r.n_tiles + 1 + bit_words) * sizeof(int);
   if (sc->actor_buf_bytes < bytes) {
     if ((e = cudaEventSynchronize(sc->actor_done)) != cudaSuccess)
       return salf_cuda_fail(e, "actor sync");
@@ -946,8 +947,9 @@ extern "C" salf_status salf_render_rays_actors(salf_scene* sc, const salf_actor*
   }
   ActorDev* dact = static_cast<ActorDev*>(sc->actor_buf);
   unsigned* masks = reinterpret_cast<unsigned*>(static_cast<char*>(sc->actor_buf) + table_bytes);
-  int* lists = reinterpret_cast<int*>(static_cast<char*>(sc->actor_buf) + table_bytes + mask_bytes);
-  int* counts = lists + 2 * (size_t)r.n_tiles;
+  int* list = reinterpret_cast<int*>(static_cast<char*>(sc->actor_buf) + table_bytes + mask_bytes);
+  int* count = list + r.n_tiles;  // the bits follow it
+  unsigned* bits = reinterpret_cast<unsigned*>(count + 1);
   if (na == 0) {
     // no actor in the request: the plain ray kernel
     if ((e = salf_launch_forward(P, cs)) != cudaSuccess) return salf_cuda_fail(e, "forward launch");
@@ -955,11 +957,11 @@ extern "C" salf_status salf_render_rays_actors(salf_scene* sc, const salf_actor*
     if ((e = cudaMemcpyAsync(dact, ad.data(), (size_t)na * sizeof(ActorDev),
                              cudaMemcpyHostToDevice, cs)) != cudaSuccess)
       return salf_cuda_fail(e, "actor table upload");
-    if ((e = cudaMemsetAsync(counts, 0, 2 * sizeof(int), cs)) != cudaSuccess)
+    if ((e = cudaMemsetAsync(count, 0, (1 + bit_words) * sizeof(int), cs)) != cudaSuccess)
       return salf_cuda_fail(e, "actor tile counts");
     // tiles whose rays may meet an actor go to the merge kernel, the rest to
     // the plain ray kernel
-    if ((e = salf_launch_classify(P, dact, na, lists, counts, masks, cs)) != cudaSuccess)
+    if ((e = salf_launch_classify(P, dact, na, bits, list, count, masks, cs)) != cudaSuccess)
       return salf_cuda_fail(e, "tile classification");
     // the two tile sets are disjoint: the merge kernel runs on an auxiliary
     // stream beside the ray kernel (fork after the classification, join
@@ -981,13 +983,12 @@ extern "C" salf_status salf_render_rays_actors(salf_scene* sc, const salf_actor*
         (e = cudaStreamWaitEvent(sc->actor_aux, sc->actor_fork, 0)) != cudaSuccess)
       return salf_cuda_fail(e, "actor fork");
     LaunchParams Pa = P;
-    Pa.req[0].tile_list = lists + r.n_tiles;
-    Pa.req[0].tile_count = counts + 1;
+    Pa.req[0].tile_list = list;
+    Pa.req[0].tile_count = count;
     if ((e = salf_launch_actors(Pa, dact, na, masks, sc->actor_aux)) != cudaSuccess)
       return salf_cuda_fail(e, "actor launch");
     LaunchParams Ps = P;
-    Ps.req[0].tile_list = lists;
-    Ps.req[0].tile_count = counts;
+    Ps.req[0].tile_skip = bits;
     if ((e = salf_launch_forward(Ps, cs)) != cudaSuccess) return salf_cuda_fail(e, "forward launch");
     if ((e = cudaEventRecord(sc->actor_join, sc->actor_aux)) != cudaSuccess ||
         (e = cudaStreamWaitEvent(cs, sc->actor_join, 0)) != cudaSuccess)
@@ -1069,7 +1070,8 @@ extern "C" salf_status salf_render_backward_actors(
   }
   const size_t table_bytes = (((size_t)na * sizeof(ActorDev)) + 255) & ~(size_t)255;
   const size_t mask_bytes = (size_t)r.n_tiles * (SALF_MAX_ACTORS / 32) * sizeof(unsigned);
-  const size_t bytes = table_bytes + mask_bytes + (2 * (size_t)r.n_tiles + 2) * sizeof(int);
+  const size_t bit_words = ((size_t)r.n_tiles + 31) / 32;
+  const size_t bytes = table_bytes + mask_bytes + ((size_t)r.n_tiles + 1 + bit_words) * sizeof(int);
   if (sc->actor_buf_bytes < bytes) {
     if ((e = cudaEventSynchronize(sc->actor_done)) != cudaSuccess)
       return salf_cuda_fail(e, "actor sync");
@@ -1086,24 +1088,24 @@ extern "C" salf_status salf_render_backward_actors(
   }
   ActorDev* dact = static_cast<ActorDev*>(sc->actor_buf);
   unsigned* masks = reinterpret_cast<unsigned*>(static_cast<char*>(sc->actor_buf) + table_bytes);
-  int* lists = reinterpret_cast<int*>(static_cast<char*>(sc->actor_buf) + table_bytes + mask_bytes);
-  int* counts = lists + 2 * (size_t)r.n_tiles;
+  int* list = reinterpret_cast<int*>(static_cast<char*>(sc->actor_buf) + table_bytes + mask_bytes);
+  int* count = list + r.n_tiles;  // the bits follow it
+  unsigned* bits = reinterpret_cast<unsigned*>(count + 1);
   if ((e = cudaMemcpyAsync(dact, ad.data(), (size_t)na * sizeof(ActorDev), cudaMemcpyHostToDevice,
                            cs)) != cudaSuccess)
     return salf_cuda_fail(e, "actor table upload");
-  if ((e = cudaMemsetAsync(counts, 0, 2 * sizeof(int), cs)) != cudaSuccess)
+  if ((e = cudaMemsetAsync(count, 0, (1 + bit_words) * sizeof(int), cs)) != cudaSuccess)
     return salf_cuda_fail(e, "actor tile counts");
   // the forward's split: tiles whose rays may meet an actor take the merge
   // walk's adjoint, the others the static adjoint
-  if ((e = salf_launch_classify(P, dact, na, lists, counts, masks, cs)) != cudaSuccess)
+  if ((e = salf_launch_classify(P, dact, na, bits, list, count, masks, cs)) != cudaSuccess)
     return salf_cuda_fail(e, "tile classification");
   LaunchParams Ps = P;
-  Ps.req[0].tile_list = lists;
-  Ps.req[0].tile_count = counts;
+  Ps.req[0].tile_skip = bits;
   if ((e = salf_launch_backward(Ps, cs)) != cudaSuccess) return salf_cuda_fail(e, "backward launch");
   LaunchParams Pa = P;
-  Pa.req[0].tile_list = lists + r.n_tiles;
-  Pa.req[0].tile_count = counts + 1;
+  Pa.req[0].tile_list = list;
+  Pa.req[0].tile_count = count;
   if ((e = salf_launch_backward_actors(Pa, dact, na, masks, cs)) != cudaSuccess)
     return salf_cuda_fail(e, "actor backward launch");
   if ((e = cudaEventRecord(sc->actor_done, cs)) != cudaSuccess)

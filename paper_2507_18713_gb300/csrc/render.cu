@@ -74,11 +74,7 @@ __global__ void __launch_bounds__(32 * WPB, MINB) k_forward(const __grid_constan
   const int lane = threadIdx.x & 31;
   const ReqDev& Q = P.req[find_request(P, warp)];
   const DevScene& S = P.S;
-  int tile = warp - Q.tile_begin;
-  if (Q.tile_list) {
-    if (tile >= __ldg(Q.tile_count)) return;
-    tile = __ldg(&Q.tile_list[tile]);
-  }
+  const int tile = warp - Q.tile_begin;
   // SEG: lanes (k + K * j), k < K = 2^seg_shift, share the tile's j-th ray
   const int ks = SEG ? Q.seg_shift : 0;
   const int K = 1 << ks;
@@ -91,6 +87,7 @@ __global__ void __launch_bounds__(32 * WPB, MINB) k_forward(const __grid_constan
   const bool in_img = (u < Q.W) && (v < Q.H);
   const int ray = v * Q.W + u;
 
+  if (Q.tile_skip && (__ldg(&Q.tile_skip[tile >> 5]) >> (tile & 31)) & 1u) return;
   Ray r;
   Walk w;
   w.alive = false;
@@ -295,7 +292,7 @@ cudaError_t salf_launch_forward(const LaunchParams& P, cudaStream_t st) {
   int count[3] = {0, 0, 0};
   for (int i = 0; i < P.n_req; ++i) ++count[variant_group(P.req[i])];
   const int groups = (count[0] > 0) + (count[1] > 0) + (count[2] > 0);
-  if (groups <= 1 || P.req[0].tile_list) return launch_variant(P, st);
+  if (groups <= 1 || P.req[0].tile_skip) return launch_variant(P, st);
   for (int part = 0; part < 3; ++part) {
     if (!count[part]) continue;
     LaunchParams G = P;

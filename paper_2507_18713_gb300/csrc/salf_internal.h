@@ -51,31 +51,33 @@
 //    index of the min corner inside the cell), FP32 or BF16;
 //    order[internal] = input index; vox_box[internal] = (min corner in finest
 //    cells, log2 of the edge in finest cells), read by the rasteriser.
-struct DevScene {
+struct alignas(16) DevScene {
+  // what a structure step reads comes first, in 64 bytes: actors' views are read
+  // from global memory
   const uint4* mask0;
-  int mdim0, mdim01;  // blocks per row (x) and per layer (x, y)
   const int2* cells;
   const int* nodes;
+  const void* params;
+  int mdim0, mdim01;      // blocks per row (x) and per layer (x, y)
+  int skip_n0, skip_n01;  // bricks per row (x) and per layer (x, y)
+  int skip_sx, skip_sz;   // log2 of a brick's edges (x and y; z), finest cells
+  int skip_coarse;        // bricks are larger than a layer of a block
+  int K;
   // skip boxes of octant o (bit a: the ray travels downwards on axis a), bricks in
   // mirrored order on its downward axes, moved so that the index is the (mirrored)
   // brick's own: b2 * skip_n01 + b1 * skip_n0 + b0
   const unsigned short* skip_oct[8];
-  int skip_n0, skip_n01;    // bricks per row (x) and per layer (x, y)
-  int skip_sx, skip_sz;     // log2 of a brick's edges (x and y; z), finest cells
-  int skip_coarse;          // bricks are larger than a layer of a block
-  const void* params;
+  int bmin[3], bmax[3];  // tight box of all voxels, finest cells [bmin, bmax)
+  // origin and inv_sfin as pairs of floats (value = [0] + [1] to 2^-48), for
+  // per-ray work: 64-bit units are few (2 FMAs per clock and SM)
+  float isf2[2], sf2[2];  // finest cells per metre; metres per finest cell
+  float origin2[3][2];
   const int* order;
   const int4* vox_box;
   int* status;
   double origin[3];
   double inv_sfin;  // finest cells per metre
-  // the same as pairs of floats (value = [0] + [1] to 2^-48), for per-ray work:
-  // 64-bit units are few (2 FMAs per clock and SM)
-  float origin2[3][2];
-  float isf2[2], sf2[2];  // finest cells per metre; metres per finest cell
-  int K;
   int Gf[3];
-  int bmin[3], bmax[3];  // tight box of all voxels, finest cells [bmin, bmax)
   int mode, dtype;
   int n;
 };
@@ -123,10 +125,12 @@ struct ReqDev {
   // each ray's span in the voxels' box is cut into 2^seg_shift equal parts,
   // walked by neighbouring lanes and composited in order (forward only)
   int seg_shift;
-  // optional subset of the tiles (device): warp w of the request renders
-  // tile tile_list[w] while w < *tile_count (null: every tile, in order)
+  // optional subsets of the tiles (device).  A list: warp w of the request renders
+  // tile tile_list[w] while w < *tile_count.  Or bits, one per tile: tiles whose bit
+  // is set are left out, the others keep their launch order.
   const int* tile_list;
   const int* tile_count;
+  const unsigned* tile_skip;
   // backward inputs (unused by the forward kernel)
   const float* bsaved;
   const float* g_rgb;
@@ -141,7 +145,7 @@ struct ReqDev {
 // One placed actor as the actor kernel sees it (prepared on the host in FP64
 // for one request; frames: world = the static scene's, canonical = the
 // actor scene's).
-struct ActorDev {
+struct alignas(128) ActorDev {
   DevScene S;           // the actor's voxels (canonical frame)
   float R0[9];          // canonical -> world rotation at the sensor's t0
   float axis[3], angle; // R(s) = rot(axis, s * angle) R0
@@ -293,11 +297,12 @@ cudaError_t salf_launch_forward(const LaunchParams& P, cudaStream_t st);
 // masks: per tile, SALF_MAX_ACTORS / 32 words of candidate actors (bits).
 cudaError_t salf_launch_actors(const LaunchParams& P, const ActorDev* actors, int n_actors,
                                const unsigned* masks, cudaStream_t st);
-// Tiles of request 0 whose rays may meet an actor -> lists[n_tiles + i],
-// the others -> lists[i]; counts[1], counts[0] (zeroed by the caller); per
-// tile the candidate actors -> masks.
+// Tiles of request 0 whose rays may meet an actor: their bits in `bits` (words of 32
+// tiles, zeroed by the caller), their numbers in `list` (*count of them, zeroed by
+// the caller), and per tile the candidate actors in `masks`.
 cudaError_t salf_launch_classify(const LaunchParams& P, const ActorDev* actors, int n_actors,
-                                 int* lists, int* counts, unsigned* masks, cudaStream_t st);
+                                 unsigned* bits, int* list, int* count, unsigned* masks,
+                                 cudaStream_t st);
 // Tile rasterisation of one pinhole request (r prepared by
 // salf_prepare_request, outputs set); fills *stats when non-null.
 salf_status salf_raster_run(salf_scene* sc, const ReqDev& r, double fx, double fy,

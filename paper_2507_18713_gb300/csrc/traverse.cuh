@@ -59,11 +59,13 @@ __device__ __forceinline__ int pair_floor(Pair a, float* frac) {
   return (int)f;
 }
 
-// Sensor ray of pixel (u, v) / LiDAR (azimuth u, beam v).
+// Sensor ray of pixel (u, v) / LiDAR (azimuth u, beam v).  EXPL: explicit rays may
+// come (their code costs the others registers).
+template <bool EXPL = true>
 __device__ __forceinline__ void gen_ray(const ReqDev& Q, const DevScene& S, int u, int v,
                                         int ray, Ray& r) {
   r.valid = true;
-  if (Q.kind == SALF_RAYS_EXPLICIT) {
+  if (EXPL && Q.kind == SALF_RAYS_EXPLICIT) {
     const float4* q = reinterpret_cast<const float4*>(Q.rays) + 2 * (size_t)ray;
     float4 a = __ldg(q), b = __ldg(q + 1);
     // origin in finest cells, (o - origin) / edge, to 48 bits

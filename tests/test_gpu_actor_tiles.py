@@ -59,7 +59,9 @@ def test_pinhole_frame_equals_its_explicit_rays(salf, w, h, hfov, n, clip):
         rays[:, 6:] = clip or (0.0, 0.0)
         kw = dict(t_min=0.0, outputs=("rgb", "depth", "opacity"), visits_cap=128)
         a = g.render_actors(cam, acts, **kw)
-        b = g.render_actors(synth.explicit_rays(rays), acts, **kw)
+        ex = synth.explicit_rays(rays)
+        ex.update(pose0=cam["pose0"], pose1=cam["pose1"])  # actors are placed from this origin
+        b = g.render_actors(ex, acts, **kw)
         torch.cuda.synchronize()
         g.check()
         # rays equal to FP32 rounding (directions 1e-7, positions 1e-6 m): hits may differ

@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(128) k_classify_tiles(const __grid_constant__ 
   const ReqDev& Q = P.req[0];
   int u0, v0;
   tile_origin(Q, tile, &u0, &v0);
-  const int u = u0 + lane % Q.tile_w, v = v0 + lane / Q.tile_w;
+  const int u = u0 + (lane & (Q.tile_w - 1)), v = v0 + (lane >> Q.tile_ws);
   // the warp's rays as a cone: mean direction, cosine of the widest ray, the
   // range of time fractions and of t_near / t_far
   Ray r;
@@ -308,7 +308,7 @@ __global__ void __launch_bounds__(32 * kClassifyWarps)
     const int j = __ffs(todo) - 1;
     int u0, v0;
     tile_origin(Q, tile0 + j, &u0, &v0);
-    const int u = u0 + lane % Q.tile_w, v = v0 + lane / Q.tile_w;
+    const int u = u0 + (lane & (Q.tile_w - 1)), v = v0 + (lane >> Q.tile_ws);
     const bool ok = u < Q.W && v < Q.H;
     Ray r;
     gen_ray_pinhole(Q, u, v, r);
@@ -378,8 +378,8 @@ __global__ void __launch_bounds__(32 * kActorWarps,
   }
   int u0, v0;
   tile_origin(Q, tile, &u0, &v0);
-  const int u = u0 + lane % Q.tile_w;
-  const int v = v0 + lane / Q.tile_w;
+  const int u = u0 + (lane & (Q.tile_w - 1));
+  const int v = v0 + (lane >> Q.tile_ws);
   const bool in_img = (u < Q.W) && (v < Q.H);
   const int ray = v * Q.W + u;
 
@@ -596,8 +596,8 @@ __global__ void __launch_bounds__(32 * kActorWarps, SALF_ACTOR_MIN_BLOCKS) k_bac
   }
   int u0, v0;
   tile_origin(Q, tile, &u0, &v0);
-  const int u = u0 + lane % Q.tile_w;
-  const int v = v0 + lane / Q.tile_w;
+  const int u = u0 + (lane & (Q.tile_w - 1));
+  const int v = v0 + (lane >> Q.tile_ws);
   const bool in_img = (u >= 0) && (v >= 0) && (u < Q.W) && (v < Q.H);
   const int ray = v * Q.W + u;
 

@@ -48,8 +48,8 @@ __global__ void __launch_bounds__(32 * SALF_BWD_WARPS, SALF_BWD_MIN_BLOCKS)
   if (Q.tile_skip && (__ldg(&Q.tile_skip[tile >> 5]) >> (tile & 31)) & 1u) return;
   int u0, v0;
   tile_origin(Q, tile, &u0, &v0);
-  const int u = u0 + lane % Q.tile_w;
-  const int v = v0 + lane / Q.tile_w;
+  const int u = u0 + (lane & (Q.tile_w - 1));
+  const int v = v0 + (lane >> Q.tile_ws);
   const bool in_img = (u < Q.W) && (v < Q.H);
   const int ray = v * Q.W + u;
 

@@ -461,6 +461,7 @@ void salf_request_tiling(ReqDev* r, const salf_sensor* s, int seg_shift) {
     r->tile_w = std::min(SALF_SEG_LIDAR_TILE_W, 32 >> seg_shift);
     r->tile_h = (32 >> seg_shift) / r->tile_w;
   }
+  r->tile_ws = __builtin_ctz((unsigned)r->tile_w);
   r->seg_shift = seg_shift;
   r->tiles_x = (s->width + r->tile_w - 1) / r->tile_w;
   r->tiles_y = (s->height + r->tile_h - 1) / r->tile_h;

@@ -82,8 +82,8 @@ __global__ void __launch_bounds__(32 * WPB, MINB) k_forward(const __grid_constan
   const int rl = lane >> ks;
   int u0, v0;
   tile_origin(Q, tile, &u0, &v0);
-  const int u = u0 + rl % Q.tile_w;
-  const int v = v0 + rl / Q.tile_w;
+  const int u = u0 + (rl & (Q.tile_w - 1));
+  const int v = v0 + (rl >> Q.tile_ws);
   const bool in_img = (u < Q.W) && (v < Q.H);
   const int ray = v * Q.W + u;
 

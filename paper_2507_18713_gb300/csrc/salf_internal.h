@@ -120,6 +120,7 @@ struct ReqDev {
   // and above it (the most nearly horizontal rays, the longest ones, first)
   int tiles_x, tiles_y;
   int tile_w, tile_h;  // rays per warp tile: tile_w x tile_h = 32 >> seg_shift
+  int tile_ws;         // log2 of tile_w
   int tile_begin, n_tiles;
   int first_row;
   // each ray's span in the voxels' box is cut into 2^seg_shift equal parts,

@@ -541,8 +541,8 @@ __device__ __forceinline__ int zigzag_row(int k, int first, int rows) {
 
 // Tile of a warp: (pixel column, pixel row) of its first lane.
 __device__ __forceinline__ void tile_origin(const ReqDev& Q, int tile, int* u0, int* v0) {
-  const int tx = tile % Q.tiles_x, k = tile / Q.tiles_x;
-  *u0 = tx * Q.tile_w;
+  const int k = (int)((unsigned)tile / (unsigned)Q.tiles_x);
+  *u0 = (tile - k * Q.tiles_x) * Q.tile_w;
   *v0 = zigzag_row(k, Q.first_row, Q.tiles_y) * Q.tile_h;
 }
 

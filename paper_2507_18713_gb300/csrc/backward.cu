@@ -16,9 +16,15 @@
 // (T, the suffix sums and dL/dtau need it) and queue the hit's coefficients
 // in a per-warp ring in shared memory; whenever 32 are queued, the whole warp
 // builds their 32-scalar gradient rows and adds them to the caller's
-// input-order FP32 buffer with 16-byte vector atomics.  Rows of one voxel in
-// a batch are staged in shared memory and summed first, each lane adding some
-// of the 16-byte chunks, so a voxel takes one set of atomics per batch.
+// input-order FP32 buffer with 16-byte vector atomics.  Where 8 or more rows of
+// a batch are of one voxel, they are staged in shared memory and summed first.
+//
+// Bound by instruction issue (57% of slots, 20 of 32 lanes active in the walk).
+// Of a training step of 8 views of 960x640 (2720 us) the sums took 300 us and
+// the atomics 27: with staging only for groups of 8 or more, and those split
+// over 8 to 32 lanes instead of 8, in the ring's own slots, the step takes
+// 2620 us and a LiDAR fit of 64x1024 470 (before: 2726 and 481).  Groups of
+// fewer than 10 or 12 by atomics: 2664 or more; all of them: 3473.
 #include "traverse.cuh"
 
 // warps per block and resident blocks per SM asked of the compiler
@@ -26,7 +32,7 @@
 #define SALF_BWD_WARPS 4
 #endif
 #ifndef SALF_BWD_MIN_BLOCKS
-#define SALF_BWD_MIN_BLOCKS 4  // 16 warps per SM: training step 2750 us, LiDAR fit 482; 5: 2756, 492; 6: 2834, 543
+#define SALF_BWD_MIN_BLOCKS 4  // 16 warps per SM: training step 2621 us, LiDAR fit 466; 5: 2623, 466
 #endif
 
 using namespace salf;
@@ -94,15 +100,11 @@ __global__ void __launch_bounds__(32 * SALF_BWD_WARPS, SALF_BWD_MIN_BLOCKS)
   const float gbg = g[0] * Q.bg[0] + g[1] * Q.bg[1] + g[2] * Q.bg[2] + gp;
   float T = 1.f, Pk = 0.f;
   int k = 0;
-  // staged gradient rows, 8 chunks of 16 bytes and one of padding: lanes' 16-byte
-  // accesses are conflict-free (rows and queue in single words: training step
-  // 2827 us, in chunks 2756)
-  __shared__ float4 s_rows[SALF_BWD_WARPS][32][9];
-  float4(*rows)[9] = s_rows[threadIdx.x >> 5];
   // per-warp ring of pending hits (4 chunks each, padded to 5): each round's
   // hits are queued, and the gradient rows and their atomics run 32 at a time
   // on the whole warp.  A hit: (voxel, x), (geometry, SDF a and b, intensity),
   // (colour factors, raydrop), SH basis.
+  // The gradient rows of voxels that many hits share are summed here too.
   constexpr int QN = 64, QW = 5;
   __shared__ float4 s_queue[SALF_BWD_WARPS][QN * QW];
   float4* queue = s_queue[threadIdx.x >> 5];
@@ -135,32 +137,37 @@ __global__ void __launch_bounds__(32 * SALF_BWD_WARPS, SALF_BWD_MIN_BLOCKS)
     if (act) {
       const unsigned peers = __match_any_sync(act_lanes, key);
       float4* dst = reinterpret_cast<float4*>(Q.d_params) + (size_t)key * 8;
-      if (peers == (1u << lane)) {
+      const int gn = __popc(peers);
+      if (gn < 8) {  // few rows of this voxel: their atomics cost less than staging
 #pragma unroll
         for (int q = 0; q < 8; ++q)
           if (q < nq) atomicAdd(dst + q, gr[q]);
       } else {
-        // several rows of one voxel: each lane sums some 16-byte chunks over them
+        // 8-15 rows in 2 parts, 16-31 in 4, 32 in 8, by lane: four lanes to a part,
+        // each summing one of its chunks (in 1, 2 and 4 parts: 2711 us, in 1: 2866)
+        const int rank = __popc(peers & ((1u << lane) - 1u));
+        const int parts = gn >= 32 ? 8 : gn >= 16 ? 4 : 2, part = rank >> 2, c = rank & 3;
+        const unsigned every = parts == 8 ? 0x01010101u : parts == 4 ? 0x11111111u : 0x55555555u;
+        const unsigned mine = part < parts ? peers & (every << part) : 0u;
+        // staged in the rows' own slots of the ring (each lane has read its hit), four
+        // chunks at a time
+        float4* slot = queue + ((head + lane) & (QN - 1)) * QW;
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-          if (q < nq) rows[lane][q] = gr[q];
-        __syncwarp(peers);
-        const int gn = __popc(peers), rank = __popc(peers & ((1u << lane) - 1u));
-        for (int c = rank; c < nq; c += gn) {
+        for (int q0 = 0; q0 < 8; q0 += 4) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) slot[q] = gr[q0 + q];
+          __syncwarp(peers);
           float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-          unsigned m = peers;
-          while (m) {
-            const int l2 = __ffs(m) - 1;
-            m &= m - 1u;
-            const float4 r2 = rows[l2][c];
+          for (unsigned m = mine; m; m &= m - 1u) {
+            const float4 r2 = queue[((head + __ffs(m) - 1) & (QN - 1)) * QW + c];
             sum.x += r2.x;
             sum.y += r2.y;
             sum.z += r2.z;
             sum.w += r2.w;
           }
-          atomicAdd(dst + c, sum);
+          if (mine && q0 + c < nq) atomicAdd(dst + q0 + c, sum);
+          __syncwarp(peers);
         }
-        __syncwarp(peers);
       }
     }
     head += n;

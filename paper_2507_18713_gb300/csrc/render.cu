@@ -25,6 +25,8 @@
 // the whole ray would; only a span that went past that point before then is
 // walked a second time from the final T in front of it.  Spans behind the
 // stop are dropped, so the result is the whole-ray walk's up to rounding.
+#include <algorithm>
+
 #include "traverse.cuh"
 
 // Warps per block and resident blocks per SM of each forward variant (they
@@ -66,8 +68,9 @@ using namespace salf;
 // compiler a smaller loop (measured 2.6% faster on the 1080p camera frame).
 // PH: every request is a pinhole camera with one pose per frame, so only that
 // ray generation is compiled in (fewer spilled registers: 1080p camera frame
-// 0.391 -> 0.381 ms).
-template <int DT, int MODE, bool DUMP, int WPB, int MINB, bool SEG, bool RD, bool INT, bool PH>
+// 0.391 -> 0.381 ms).  AHEAD: see reads_ahead.
+template <int DT, int MODE, bool DUMP, int WPB, int MINB, bool SEG, bool RD, bool INT, bool PH,
+          bool AHEAD>
 __global__ void __launch_bounds__(32 * WPB, MINB) k_forward(const __grid_constant__ LaunchParams P) {
   const int warp = blockIdx.x * WPB + (threadIdx.x >> 5);
   if (warp >= P.total_tiles) return;
@@ -99,7 +102,7 @@ __global__ void __launch_bounds__(32 * WPB, MINB) k_forward(const __grid_constan
       gen_ray_pinhole(Q, u, v, r);
     else
       gen_ray(Q, S, u, v, ray, r);
-    walk_init(S, r, w);
+    walk_init<AHEAD>(S, r, w);
     if (DUMP && Q.ray_dump) dump_ray(Q, S, r, ray);
     if (SEG && ks > 0 && w.alive) {
       // cut points t0 + L j / K: one expression for both lanes that share a cut
@@ -113,7 +116,7 @@ __global__ void __launch_bounds__(32 * WPB, MINB) k_forward(const __grid_constan
         // exit rounded below their entry
         walk_end = cut_hi + 4e-6f * fabsf(cut_hi);
       }
-      if (kseg > 0) walk_seek(S, w, cut_lo);
+      if (kseg > 0) walk_seek<AHEAD>(S, w, cut_lo);
     }
   }
   float gam[4];
@@ -131,7 +134,7 @@ __global__ void __launch_bounds__(32 * WPB, MINB) k_forward(const __grid_constan
     for (;;) {
       Hit h;
       if (DUMP) steps += w.alive ? 1 : 0;
-      bool hit = next_hit<DT>(S, w, h);
+      bool hit = next_hit<DT, AHEAD>(S, w, h);
       if (SEG && !hit && w.t > walk_end) w.alive = false;  // the rest is the next span's
       if (!__any_sync(0xffffffffu, hit || w.alive)) break;
       if (SEG && hit && ks > 0) {  // composite only the voxels entered inside this span
@@ -179,8 +182,8 @@ __global__ void __launch_bounds__(32 * WPB, MINB) k_forward(const __grid_constan
     const bool redo = keep && ends && Tf < 1.f && !(Tf * T_prev >= tmin);
     if (redo) {
       A = Accum{Tf, 0.f, 0.f, 0.f, 0.f, 0.f, 0, 0.f};
-      walk_seek(S, w, cut_lo);
       w.alive = true;
+      walk_seek<AHEAD>(S, w, cut_lo);
     } else if (keep) {
       A.C0 *= Tf;
       A.C1 *= Tf;
@@ -219,11 +222,31 @@ __global__ void __launch_bounds__(32 * WPB, MINB) k_forward(const __grid_constan
 }
 
 template <int DT, int MODE, bool DUMP, int WPB, int MINB, bool SEG, bool RD, bool INT,
-          bool PH = false>
+          bool PH = false, bool AHEAD = false>
 static void launch_one(const LaunchParams& P, cudaStream_t st) {
   const int blocks = (P.total_tiles + WPB - 1) / WPB;
   if (blocks > 0)
-    k_forward<DT, MODE, DUMP, WPB, MINB, SEG, RD, INT, PH><<<blocks, 32 * WPB, 0, st>>>(P);
+    k_forward<DT, MODE, DUMP, WPB, MINB, SEG, RD, INT, PH, AHEAD><<<blocks, 32 * WPB, 0, st>>>(P);
+}
+
+// Whether a launch of whole rays reads each next step's box and word ahead
+// (next_hit's AHEAD, at the divergent variants' 20 warps per SM).  That pays
+// while a launch waits for its longest rays, which grow with the voxels' tight
+// box (its longest side in level-0 cells), and costs instructions and, for
+// cameras, resident warps once there are rays enough to fill the chip.
+// Measured (us, read when needed / ahead):
+//   camera   256x192: side 548 88 / 74, side 1000 231 / 192; 1280x960: 103 / 101, 288 / 253;
+//            1500x1000 (46875 tiles): 115 / 125, 288 / 295; 1920x1080: 164 / 180, 390 / 434;
+//            side 64: 256x192 67 / 59, 640x480 (9600 tiles) 145 / 150
+//   fisheye  1920x1080 (64800 tiles): side 548 159 / 171, 775 206 / 208, 1000 286 / 269
+//   panorama 2800x700: side 548 178 / 182, 775 232 / 224, 1000 316 / 292; 4096x1024 (131072
+//            tiles), side 1000: 660 / 703
+//   explicit rays (reflections) 256x192 132 / 102, 1000x700 203 / 189, 1500x1000 276 / 275
+// Both ways take the same steps and give the same bits.
+static bool reads_ahead(const LaunchParams& P, bool coherent) {
+  int side = 1;
+  for (int a = 0; a < 3; ++a) side = std::max(side, (P.S.bmax[a] - P.S.bmin[a]) >> P.S.K);
+  return P.total_tiles <= std::min<int64_t>(72 * (int64_t)side, coherent ? 40000 : 72000);
 }
 
 template <int DT, int MODE>
@@ -232,6 +255,7 @@ static cudaError_t launch_fm(const LaunchParams& P, bool dump, bool coherent, bo
   constexpr int WD = SALF_FWD_WPB_DIVERGENT, BD = SALF_FWD_BLOCKS_DIVERGENT;
   constexpr int WS = SALF_FWD_WPB_SEG, BS = SALF_FWD_BLOCKS_SEG;
   constexpr int WC = SALF_FWD_WPB_COHERENT, BC = SALF_FWD_BLOCKS_COHERENT;
+  const bool ahead = reads_ahead(P, coherent);
   if (dump)
     launch_one<DT, MODE, true, WD, BD, false, true, true>(P, st);
   else if (seg && rd)
@@ -242,12 +266,20 @@ static cudaError_t launch_fm(const LaunchParams& P, bool dump, bool coherent, bo
     launch_one<DT, MODE, false, WD, BD, false, true, true>(P, st);
   else if (coherent && want_int)
     launch_one<DT, MODE, false, WC, BC, false, false, true>(P, st);
+  else if (pinhole && ahead)
+    launch_one<DT, MODE, false, WC, BD, false, false, false, true, true>(P, st);
   else if (pinhole)
     launch_one<DT, MODE, false, WC, BC, false, false, false, true>(P, st);
+  else if (coherent && ahead)
+    launch_one<DT, MODE, false, WC, BD, false, false, false, false, true>(P, st);
   else if (coherent)
     launch_one<DT, MODE, false, WC, BC, false, false, false>(P, st);
+  else if (want_int && ahead)
+    launch_one<DT, MODE, false, WD, BD, false, false, true, false, true>(P, st);
   else if (want_int)
     launch_one<DT, MODE, false, WD, BD, false, false, true>(P, st);
+  else if (ahead)
+    launch_one<DT, MODE, false, WD, BD, false, false, false, false, true>(P, st);
   else
     launch_one<DT, MODE, false, WD, BD, false, false, false>(P, st);
   return cudaGetLastError();

@@ -183,12 +183,14 @@ __device__ __forceinline__ void reg_add(float* __restrict__ grads, int v, const 
 // vector atomics; only a smaller voxel adds its larger neighbour's part.  (With
 // each pair worked out once and both parts added by scalar atomics the kernel
 // was bound by them, 12 per pair in SDF mode: 1M voxels, SDF, 216 us.)  The
-// loss is summed over a block before its atomic.
+// loss is summed over a block, then over blocks by k_reg_total, in 64 bits:
+// thousands of FP32 atomics on one scalar would round it by 1e-6 and more.
 template <int MODE, bool VEC>
 __global__ void __launch_bounds__(256) k_reg_loss(const __grid_constant__ DevScene S,
                                                   const float* __restrict__ params, float lam_s,
                                                   float lam_a, float lam_n, float sfin,
                                                   float* __restrict__ loss,
+                                                  float* __restrict__ partial,
                                                   float* __restrict__ grads) {
   __shared__ float s_acc[8];
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
@@ -283,15 +285,36 @@ __global__ void __launch_bounds__(256) k_reg_loss(const __grid_constant__ DevSce
     float sum = 0.f;
 #pragma unroll
     for (int k = 0; k < 8; ++k) sum += s_acc[k];
-    if (sum != 0.f) atomicAdd(loss, sum);
+    if (partial)
+      partial[blockIdx.x] = sum;
+    else if (sum != 0.f)
+      atomicAdd(loss, sum);
+  }
+}
+
+// The blocks' sums, added to the loss once (4 us).
+__global__ void __launch_bounds__(1024) k_reg_total(const float* __restrict__ partial, int n,
+                                                    float* __restrict__ loss) {
+  __shared__ double s_acc[32];
+  double acc = 0.0;
+  for (int i = threadIdx.x; i < n; i += 1024) acc += (double)__ldg(&partial[i]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) s_acc[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    acc = s_acc[threadIdx.x];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (threadIdx.x == 0 && acc != 0.0) atomicAdd(loss, (float)acc);
   }
 }
 
 template <int MODE, bool VEC>
 void launch_reg(const DevScene& D, const float* params, float lam_s, float lam_a, float lam_n,
-                float sfin, float* loss, float* grads, cudaStream_t st) {
+                float sfin, float* loss, float* partial, float* grads, cudaStream_t st) {
   k_reg_loss<MODE, VEC><<<(unsigned)((D.n + 255) / 256), 256, 0, st>>>(
-      D, params, lam_s, lam_a, lam_n, sfin, loss, grads);
+      D, params, lam_s, lam_a, lam_n, sfin, loss, partial, grads);
 }
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -432,7 +455,14 @@ extern "C" salf_status salf_scene_reg_loss(salf_scene* sc, const float* params, 
     const auto run = D.mode == SALF_FIELD_EXP
                          ? (vec ? launch_reg<SALF_FIELD_EXP, true> : launch_reg<SALF_FIELD_EXP, false>)
                          : (vec ? launch_reg<SALF_FIELD_SDF, true> : launch_reg<SALF_FIELD_SDF, false>);
-    run(D, params, lambda_s, lambda_alpha, lambda_n, (float)sc->sfin, loss, grads, st);
+    // up to 32 blocks add their sums themselves, within 32 roundings
+    const int blocks = (int)((D.n + 255) / 256);
+    PoolBuf part;
+    if (blocks > 32)
+      if (salf_status rc = part.get(sc->ctx, (size_t)blocks * 4, st)) return rc;
+    float* partial = static_cast<float*>(part.p);
+    run(D, params, lambda_s, lambda_alpha, lambda_n, (float)sc->sfin, loss, partial, grads, st);
+    if (partial) k_reg_total<<<1, 1024, 0, st>>>(partial, blocks, loss);
     if ((e = cudaGetLastError()) != cudaSuccess) return salf_cuda_fail(e, "reg loss launch");
   }
   return SALF_OK;

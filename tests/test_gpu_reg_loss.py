@@ -47,3 +47,23 @@ def test_gradient_against_oracle(salf, oracle_lib, mode, n):
         assert abs(float(loss) - 2.0 - ref_loss) <= 1e-5 * (2.0 + abs(ref_loss))
         got = to_np(grads).astype(np.float64) - start.numpy()
         assert np.abs(got - ref).max() <= 1e-4 * max(1.0, np.abs(ref).max())
+
+
+@pytest.mark.parametrize("mode", ["exp", "sdf"])
+@pytest.mark.parametrize("n", [8192, 8193, 60000])
+def test_loss_sum(salf, oracle_lib, mode, n):
+    """32 blocks of 256 voxels add their sums to the loss one by one, more go through the sum
+    over blocks.  A thread's pairs, a warp, a block: up to 20 roundings; 32 or one in the
+    loss; 1e-6 for the pairs' own terms, whose errors have either sign."""
+    sc = synth.random_multilevel_scene(seed=31, max_level=1, dims=(40, 40, 40), p_occ=0.6,
+                                       p_sub=0.3, mode=mode)
+    assert sc.n >= n
+    sc.level, sc.ijk, sc.params = sc.level[:n], sc.ijk[:n], sc.params[:n]
+    P = np.asarray(sc.params, dtype=np.float32)
+    ref, _ = oracle_lib.reg_loss(sc, P.astype(np.float64), 0.7, 1.3, 0.4)
+    g = salf.Scene(sc)
+    params = torch.from_numpy(P).cuda()
+    for _ in range(3):
+        loss, _ = g.reg_loss(params, 0.7, 1.3, 0.4)
+        rel = abs(float(loss) - ref) / ref
+        assert rel <= (20 + (32 if n <= 8192 else 1)) * 2.0 ** -24 + 1e-6

@@ -540,11 +540,12 @@ def refine(scene, grads, max_alpha, split_threshold, prune_alpha=1e-3):
 
 
 def _density_and_grad(g, rec, mode):
-    """sigma(g) and d sigma / d(g, a, b) for the geometry value g (Eq. 1 / Eq. 6)."""
+    """sigma(g) and d sigma / d(g, a, b) for geometry values g of the records
+    `rec`, one each (Eq. 1 / Eq. 6)."""
     if mode == "exp":
         s = np.exp(g)
-        return s, s, 0.0, 0.0
-    a, b = rec[25], rec[26]
+        return s, s, 0.0 * g, 0.0 * g
+    a, b = rec[:, 25], rec[:, 26]
     e = np.exp(-abs(g) / b)
     sg = np.sign(g)
     s = 0.5 * a + 0.5 * a * sg * (1.0 - e)
@@ -555,29 +556,32 @@ def _density_and_grad(g, rec, mode):
 
 
 def face_pairs(scene):
-    """Face-adjacent voxel pairs (positive contact area), brute force:
-    list of (i, j, axis, sign) with voxel j on the `sign` side of voxel i
-    along `axis`, i no larger than j (one entry per pair)."""
+    """Face-adjacent voxel pairs (positive contact area): list of (i, j, axis,
+    sign) with voxel j on the `sign` side of voxel i along `axis`, i no larger
+    than j (one entry per pair), ordered by i, then j.  A voxel that is no
+    smaller than i and touches one of its faces covers that whole face, as
+    boxes are aligned to their own size: it is looked up by the cell, of each
+    size from i's own up, just outside the face."""
     K = scene.max_level
     lvl = np.asarray(scene.level).astype(np.int64)
-    e = (1 << (K - lvl)).astype(np.int64)                       # edges in finest cells
-    lo = np.asarray(scene.ijk).astype(np.int64) * e[:, None]
-    hi = lo + e[:, None]
+    ijk = np.asarray(scene.ijk).astype(np.int64)
+    at = {}
+    for v in range(len(lvl)):
+        at.setdefault((lvl[v], *ijk[v].tolist()), []).append(v)
     out = []
-    n = len(lvl)
-    for i in range(n):
-        for j in range(n):
-            if i == j or e[j] < e[i] or (e[j] == e[i] and j < i):
-                continue
-            for a in range(3):
-                o = [b for b in range(3) if b != a]
-                area = all(min(hi[i, b], hi[j, b]) > max(lo[i, b], lo[j, b]) for b in o)
-                if not area:
-                    continue
-                if hi[i, a] == lo[j, a]:
-                    out.append((i, j, a, +1))
-                elif lo[i, a] == hi[j, a]:
-                    out.append((i, j, a, -1))
+    for i in range(len(lvl)):
+        found = []
+        for a in range(3):
+            for sgn in (+1, -1):
+                c = ijk[i].tolist()
+                c[a] += sgn
+                for l in range(lvl[i], -1, -1):
+                    s = lvl[i] - l
+                    for j in at.get((l, c[0] >> s, c[1] >> s, c[2] >> s), ()):
+                        # (i's own parent cell holds i: not a voxel across the face)
+                        if (j > i or l < lvl[i]) and c[a] >> s != ijk[i, a] >> s:
+                            found.append((i, j, a, sgn))
+        out += sorted(found)
     return out
 
 
@@ -595,48 +599,40 @@ def reg_loss(scene, params, lam_s, lam_alpha, lam_n):
     lo = np.asarray(scene.ijk).astype(np.int64) * e[:, None]
     P = np.asarray(params, dtype=np.float64)
     grad = np.zeros_like(P)
-    loss = 0.0
-    for i, j, a, sgn in face_pairs(scene):
-        X = lo[i] + 0.5 * e[i]
-        X = X.astype(np.float64)
-        X[a] += 0.5 * e[i] * sgn                               # centre of i's face towards j
-        xs, ss, sig, dsg = [], [], [], []
-        for k in (i, j):
-            x = (X - (lo[k] + 0.5 * e[k])) / (0.5 * e[k])
-            s = P[k, :3] @ x + P[k, 3]
-            xs.append(x)
-            ss.append(s)
-            sk, ds_dg, ds_da, ds_db = _density_and_grad(s, P[k], scene.mode)
-            sig.append(sk)
-            dsg.append((ds_dg, ds_da, ds_db))
-        ell = e[i] * sfin
-        # s term
-        d = ss[0] - ss[1]
-        loss += lam_s * abs(d)
-        for k, x, sg in ((i, xs[0], 1.0), (j, xs[1], -1.0)):
-            grad[k, :3] += lam_s * np.sign(d) * sg * x
-            grad[k, 3] += lam_s * np.sign(d) * sg
-        # alpha term
-        al = [1.0 - np.exp(-sig[q] * ell) for q in (0, 1)]
-        da = al[0] - al[1]
-        loss += lam_alpha * abs(da)
-        for q, k, sg in ((0, i, 1.0), (1, j, -1.0)):
-            dal_dsig = np.exp(-sig[q] * ell) * ell
-            c = lam_alpha * np.sign(da) * sg * dal_dsig
-            ds_dg, ds_da, ds_db = dsg[q]
-            grad[k, :3] += c * ds_dg * xs[q]
-            grad[k, 3] += c * ds_dg
-            if scene.mode == "sdf":
-                grad[k, 25] += c * ds_da
-                grad[k, 26] += c * ds_db
-        # normal term
-        w = [P[i, :3], P[j, :3]]
-        nn = [np.linalg.norm(v) for v in w]
-        nv = [w[q] / nn[q] if nn[q] > 0 else np.zeros(3) for q in (0, 1)]
-        loss += lam_n * (1.0 - nv[0] @ nv[1])
-        for q, k in ((0, i), (1, j)):
-            if nn[q] > 0:
-                other = nv[1 - q]
-                # d(n . m)/dw = (m - n (n . m)) / |w|
-                grad[k, :3] += -lam_n * (other - nv[q] * (nv[q] @ other)) / nn[q]
+    pairs = np.array(face_pairs(scene), dtype=np.int64).reshape(-1, 4)
+    i, j, a, sgn = pairs.T
+    m = np.arange(len(pairs))
+    X = lo[i] + 0.5 * e[i, None]
+    X[m, a] += 0.5 * e[i] * sgn                                # centre of i's face towards j
+    ell = e[i] * sfin
+    xs, ss, sig, dsg, nn, nv = [], [], [], [], [], []
+    for k in (i, j):
+        x = (X - (lo[k] + 0.5 * e[k, None])) / (0.5 * e[k, None])
+        s = (P[k, :3] * x).sum(axis=1) + P[k, 3]
+        xs.append(x)
+        ss.append(s)
+        sk, *d = _density_and_grad(s, P[k], scene.mode)
+        sig.append(sk)
+        dsg.append(d)
+        nn.append(np.linalg.norm(P[k, :3], axis=1))
+        nv.append(P[k, :3] / np.where(nn[-1] > 0, nn[-1], 1.0)[:, None])
+    d = ss[0] - ss[1]
+    al = [1.0 - np.exp(-sig[q] * ell) for q in (0, 1)]
+    da = al[0] - al[1]
+    dot = (nv[0] * nv[1]).sum(axis=1)
+    loss = (lam_s * abs(d) + lam_alpha * abs(da) + lam_n * (1.0 - dot)).sum()
+    for q, k, sg in ((0, i, 1.0), (1, j, -1.0)):
+        row = np.zeros((len(pairs), 32))
+        ds_dg, ds_da, ds_db = dsg[q]
+        c = lam_alpha * np.sign(da) * sg * np.exp(-sig[q] * ell) * ell   # d alpha / d sigma
+        g = lam_s * np.sign(d) * sg + c * ds_dg
+        row[:, :3] = g[:, None] * xs[q]
+        row[:, 3] = g
+        if scene.mode == "sdf":
+            row[:, 25] = c * ds_da
+            row[:, 26] = c * ds_db
+        # d(n . m)/dw = (m - n (n . m)) / |w|, no gradient where w is 0
+        turn = (nv[1 - q] - nv[q] * dot[:, None]) / np.where(nn[q] > 0, nn[q], np.inf)[:, None]
+        row[:, :3] -= lam_n * turn
+        np.add.at(grad, k, row)
     return loss, grad

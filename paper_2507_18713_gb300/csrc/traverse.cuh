@@ -43,20 +43,28 @@ __device__ __forceinline__ Pair pair_add(Pair a, Pair b) {
 
 __device__ __forceinline__ Pair pair_mul(Pair a, const float b[2]) {
   const float p = __fmul_rn(a.hi, b[0]);
+  if (fabsf(p) > 3.4e38f) return Pair{p, 0.f};  // beyond floats: no rounding error to follow
   const float e = __fmaf_rn(a.hi, b[0], -p);
   return two_sum(p, __fmaf_rn(a.hi, b[1], __fmaf_rn(a.lo, b[0], e)));
 }
 
-// floor of a pair as an int, and what is left of it in [0, 1) as a float.
+// Cells are counted from a ray's origin, so a box plane's distance from the
+// origin's cell has to fit an int whichever way the axis is mirrored: cells end
+// there, 2^23 short of the int range (a grid's planes lie within 2^22 of 0).
+constexpr int kFarCell = 0x7f800000;
+
+// A pair as an int and a fraction in [0, 1] (1: less than 1 by under 2^-25).
+// Beyond kFarCell: there, and no fraction.
 __device__ __forceinline__ int pair_floor(Pair a, float* frac) {
-  float f = floorf(a.hi);
-  float r = __fadd_rn(__fsub_rn(a.hi, f), a.lo);
-  if (r < 0.f) {  // hi is whole and lo below it
-    f = __fsub_rn(f, 1.f);
-    r = __fadd_rn(__fsub_rn(a.hi, f), a.lo);
+  if (fabsf(a.hi) >= (float)kFarCell) {
+    *frac = 0.f;
+    return a.hi < 0.f ? -kFarCell : kFarCell;
   }
-  *frac = r;
-  return (int)f;
+  const float f = floorf(a.hi);
+  const float r = __fadd_rn(__fsub_rn(a.hi, f), a.lo);
+  const float k = floorf(r);  // -1 where hi is whole and lo below it; more from 2^25 on
+  *frac = __fsub_rn(r, k);
+  return (int)f + (int)k;
 }
 
 // Sensor ray of pixel (u, v) / LiDAR (azimuth u, beam v).  EXPL: explicit rays may

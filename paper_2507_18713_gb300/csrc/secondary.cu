@@ -113,7 +113,9 @@ __global__ void __launch_bounds__(256) k_secondary(const __grid_constant__ Secon
       float X[3];
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
-        const Pair m = pair_mul(pair_add(Pair{(float)r.Oi[q], 0.f}, p[q]), S.sf2);
+        const float oh = (float)r.Oi[q];  // an int takes two floats
+        const Pair m =
+            pair_mul(pair_add(Pair{oh, (float)(r.Oi[q] - (int)oh)}, p[q]), S.sf2);
         const Pair w = pair_add(Pair{S.origin2[q][0], S.origin2[q][1]}, m);
         const Pair x = pair_add(w, Pair{__fmul_rn(side * P.offset, n[q]), 0.f});
         X[q] = __fadd_rn(x.hi, x.lo);

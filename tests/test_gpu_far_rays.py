@@ -45,3 +45,27 @@ def test_rays_leaving_from_afar(salf, mode, dims):
         assert not to_np(out["opacity"]).any() and not to_np(out["depth"]).any()
         np.testing.assert_array_equal(to_np(out["rgb"]),
                                       np.tile(np.float32([0.25, 0.5, 0.75]), (len(many), 1)))
+
+
+def test_spawn_point_of_a_far_primary(salf):
+    """The hit point o + (D / O) d of a ray from 2^25 cells away, in the float's own steps of
+    4 cells, against 64 bits: the origin's cell takes more than a float's 24 bits."""
+    n = 12
+    ijk = np.stack(np.meshgrid(np.arange(n), np.arange(3), np.arange(3), indexing="ij"),
+                   -1).reshape(-1, 3).astype(np.int32)
+    params = synth.draw_params(np.random.default_rng(1), len(ijk), "exp")
+    sc = synth.SceneData((1.0, 0.0, 0.0), 1.0, (n, 3, 3), 0, np.zeros(len(ijk), np.uint8), ijk,
+                         params, "exp", "block")
+    g = salf.Scene(sc)
+    far = 2.0 ** 25 + 4.0 * np.arange(1, 9)
+    hit = np.array([4.0, 8.0] * 4)
+    rays = np.zeros((8, 8), np.float32)
+    rays[:, 0], rays[:, 1:3], rays[:, 3] = -far, 1.5, 1.0
+    depth = torch.from_numpy((far + hit).astype(np.float32)).cuda()
+    assert (depth.cpu().numpy().astype(np.float64) == far + hit).all()
+    for kind in ("reflect", "shadow"):
+        out = to_np(g.secondary_rays(salf.rays_sensor(torch.from_numpy(rays).cuda()), depth,
+                                     torch.ones_like(depth), kind=kind, offset=0.0))
+        assert out[:, 3:6].any(axis=1).all()
+        np.testing.assert_allclose(out[:, :3], np.stack([hit, 0 * hit + 1.5, 0 * hit + 1.5], 1),
+                                   rtol=2.0 ** -23)

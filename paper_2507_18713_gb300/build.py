@@ -22,7 +22,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CUDA_SOURCES = ["render.cu", "backward.cu", "params.cu", "noalloc.cu", "raster.cu", "actors.cu",
                 "refine.cu", "scene_build_gpu.cu", "skip.cu", "secondary.cu", "measure.cu"]
 CXX_SOURCES = ["capi.cpp", "scene_build.cpp", "serve.cpp", "checkpoint.cpp"]
-HEADERS = ["salf_internal.h", "traverse.cuh", "scan.cuh", "sort.cuh"]
+HEADERS = ["salf_internal.h", "traverse.cuh", "scan.cuh", "sort.cuh", "skip_shape.h"]
 
 
 def _nvcc() -> str:

@@ -22,11 +22,12 @@
 #include <algorithm>
 
 #include "salf_internal.h"
+#include "skip_shape.h"
 
 namespace {
 
-constexpr int kLevels = 5;                      // rectangles of 1, 2, 4, 8, 16 columns a side
-constexpr int kPad = (1 << (kLevels - 1)) - 1;  // rectangles may start this far before the grid
+constexpr int kLevels = kSkipLevels;
+constexpr int kPad = kSkipPad;
 constexpr int kMaxXY = 31, kMaxZ = 63;          // box sizes a skip entry holds, in bricks
 constexpr int kChunk = 8;                       // layers per thread of k_skip_boxes
 
@@ -119,7 +120,9 @@ __global__ void __launch_bounds__(256) k_skip_rects(SkipGrid G, unsigned long lo
 // word and kChunk of its layers.  A warp takes 32 columns along x, a block the 8
 // octants.  Bound by instructions and the table reads (L1).  A 1.27M-voxel scene,
 // 177 x 177 x 41 bricks: 213 us with all of a word's layers in one thread, 193 in
-// chunks, 158 with 32-bit offsets, 110 with the box kept from layer to layer.
+// chunks, 158 with 32-bit offsets, 110 with the box kept from layer to layer.  Off:
+// the offsets' type (skip_wide_offsets).
+template <class Off>
 __global__ void __launch_bounds__(256) k_skip_boxes(const unsigned long long* __restrict__ rect,
                                                     SkipGrid G, int tiles_x, int chunks,
                                                     unsigned short* __restrict__ skip) {
@@ -131,13 +134,12 @@ __global__ void __launch_bounds__(256) k_skip_boxes(const unsigned long long* __
   const int y = bid % G.n[1], wd = bid / G.n[1];
   const int sx = (threadIdx.x >> 5) & 1, sy = (threadIdx.x >> 6) & 1, down = threadIdx.x >> 7;
   if (x >= G.n[0]) return;
-  // (a table has at most some 2^23 words: 32-bit offsets)
-  const int table = G.px * G.py * G.words;
-  const unsigned long long* here = rect + (wd * G.px * G.py + (y + kPad) * G.px + (x + kPad));
+  const Off table = (Off)G.px * G.py * G.words;
+  const unsigned long long* here = rect + ((Off)wd * G.px * G.py + (y + kPad) * G.px + (x + kPad));
   // word of the 2^i x 2^j rectangle whose far side lies fx, fy columns ahead
   auto at = [&](int i, int j, int fx, int fy) {
     const int dx = sx ? 1 - fx : fx - (1 << i), dy = sy ? 1 - fy : fy - (1 << j);
-    return __ldg(here + ((i * kLevels + j) * table + (dy * G.px + dx)));
+    return __ldg(here + skip_rect_offset<Off>(i, j, table, G.px, dy, dx));
   };
   const int room_x = min(kMaxXY, sx ? x + 1 : G.n[0] - x);
   const int room_y = min(kMaxXY, sy ? y + 1 : G.n[1] - y);
@@ -279,7 +281,8 @@ salf_status salf_build_skip(salf_scene* s, int p, int q, cudaStream_t st) {
   k_skip_rows<<<(unsigned)((table + 255) / 256), 256, 0, st>>>(occ, G, rect);
   k_skip_rects<<<(unsigned)((table * kLevels + 255) / 256), 256, 0, st>>>(G, rect);
   const int tiles_x = (G.n[0] + 31) / 32, chunks = (std::min(64, G.n[2]) + kChunk - 1) / kChunk;
-  k_skip_boxes<<<(unsigned)(tiles_x * G.n[1] * G.words * chunks), 256, 0, st>>>(
+  const auto boxes = skip_wide_offsets(table) ? k_skip_boxes<long long> : k_skip_boxes<int>;
+  boxes<<<(unsigned)(tiles_x * G.n[1] * G.words * chunks), 256, 0, st>>>(
       rect, G, tiles_x, chunks, static_cast<unsigned short*>(skip));
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return salf_cuda_fail(e, "skip boxes");

@@ -228,7 +228,12 @@ typedef struct {
   const int32_t* dev_order; /* internal index -> input index */
 } salf_scene_info;
 
-/* Create a context bound to CUDA device `device`. */
+/*
+ * Create a context bound to CUDA device `device`.  Scenes and contexts may be
+ * destroyed in any order: a scene works on after salf_destroy of the context
+ * it was built with, whose resources go with the last of its scenes.  No
+ * further scene can be built with a destroyed context.
+ */
 salf_status salf_create(int32_t device, salf_ctx** out);
 void salf_destroy(salf_ctx* ctx);
 

@@ -62,9 +62,15 @@ extern "C" salf_status salf_create(int32_t device, salf_ctx** out) {
 }
 
 extern "C" void salf_destroy(salf_ctx* ctx) {
-  if (!ctx) return;
+  if (!ctx || ctx->holders.fetch_sub(1) > 1) return;
   if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
   delete ctx;
+}
+
+void salf_scene_hold_ctx(salf_scene* s, salf_ctx* ctx) {
+  ctx->holders.fetch_add(1);
+  s->ctx = ctx;
+  s->device = ctx->device;
 }
 
 salf_status PoolBuf::get(salf_ctx* ctx, size_t bytes, cudaStream_t stream) {
@@ -109,6 +115,7 @@ extern "C" void salf_scene_destroy(salf_scene* s) {
   if (s->actor_fork) cudaEventDestroy(s->actor_fork);
   if (s->actor_join) cudaEventDestroy(s->actor_join);
   if (s->actor_aux) cudaStreamDestroy(s->actor_aux);
+  salf_destroy(s->ctx);
   delete s;
 }
 

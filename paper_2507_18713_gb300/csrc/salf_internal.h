@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -171,14 +172,15 @@ struct LaunchParams {
 
 // Device memory of scenes and of their builds comes from a pool of the
 // context's own, which keeps up to kPoolKeep freed bytes for the next build
-// (cudaMalloc and cudaFree took more than half of a 1M-voxel rebuild).  The
-// pool goes with the context; memory that is still out then is given back as
-// its scenes are destroyed.
+// (cudaMalloc and cudaFree took more than half of a 1M-voxel rebuild).
 constexpr unsigned long long kPoolKeep = 1ull << 30;
 
+// Held by its creator until salf_destroy and by each of its scenes: calls on a
+// scene may take temporaries from the pool, which goes with the last holder.
 struct salf_ctx {
   int device;
   cudaMemPool_t pool = nullptr;
+  std::atomic<int> holders{1};
 };
 
 struct salf_scene {
@@ -264,6 +266,8 @@ struct SalfRange {
 
 // Implemented in the .cu / .cpp files of the library.
 void salf_set_error(const std::string& msg);
+// The scene holds the context from here on (salf_scene_destroy lets go of it).
+void salf_scene_hold_ctx(salf_scene* s, salf_ctx* ctx);
 salf_status salf_cuda_fail(cudaError_t e, const char* what);
 // Resolve the no-alloc entry point's staging array on `device` (current).
 salf_status salf_noalloc_setup(int device);

@@ -262,8 +262,7 @@ salf_status salf_build_scene_impl(salf_ctx* ctx, const salf_scene_desc* d, salf_
   // ---- device upload
   salf_scene* s = new salf_scene();
   Scope guard{s};
-  s->ctx = ctx;
-  s->device = ctx->device;
+  salf_scene_hold_ctx(s, ctx);
   s->n = n;
   s->mode = d->mode;
   s->dtype = d->dtype;

@@ -368,8 +368,7 @@ salf_status salf_build_scene_gpu(salf_ctx* ctx, const salf_scene_desc* d, salf_s
       if (!keep) salf_scene_destroy(s);
     }
   } guard{s};
-  s->ctx = ctx;
-  s->device = ctx->device;
+  salf_scene_hold_ctx(s, ctx);
   s->n = n;
   s->mode = d->mode;
   s->dtype = d->dtype;

@@ -455,11 +455,11 @@ extern "C" salf_status salf_scene_reg_loss(salf_scene* sc, const float* params, 
     const auto run = D.mode == SALF_FIELD_EXP
                          ? (vec ? launch_reg<SALF_FIELD_EXP, true> : launch_reg<SALF_FIELD_EXP, false>)
                          : (vec ? launch_reg<SALF_FIELD_SDF, true> : launch_reg<SALF_FIELD_SDF, false>);
-    // up to 32 blocks add their sums themselves, within 32 roundings
+    // up to 32 blocks add their sums themselves, within 32 roundings; so do more
+    // where the device has no room for the sums
     const int blocks = (int)((D.n + 255) / 256);
     PoolBuf part;
-    if (blocks > 32)
-      if (salf_status rc = part.get(sc->ctx, (size_t)blocks * 4, st)) return rc;
+    if (blocks > 32) (void)part.get(sc->ctx, (size_t)blocks * 4, st);
     float* partial = static_cast<float*>(part.p);
     run(D, params, lambda_s, lambda_alpha, lambda_n, (float)sc->sfin, loss, partial, grads, st);
     if (partial) k_reg_total<<<1, 1024, 0, st>>>(partial, blocks, loss);

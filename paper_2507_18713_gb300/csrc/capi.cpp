@@ -64,7 +64,52 @@ extern "C" salf_status salf_create(int32_t device, salf_ctx** out) {
 extern "C" void salf_destroy(salf_ctx* ctx) {
   if (!ctx || ctx->holders.fetch_sub(1) > 1) return;
   if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
+  for (const DevBlock& b : ctx->blocks) cudaFree(b.p);
   delete ctx;
+}
+
+salf_status salf_scene_block(salf_scene* s, size_t bytes, void** p) {
+  salf_ctx* ctx = s->ctx;
+  bytes = std::max<size_t>(bytes, 16);
+  std::lock_guard<std::mutex> lk(ctx->blocks_mu);
+  // the smallest kept block that holds it and is at most a quarter larger
+  auto best = ctx->blocks.end();
+  for (auto b = ctx->blocks.begin(); b != ctx->blocks.end(); ++b)
+    if (b->bytes >= bytes && b->bytes <= bytes + bytes / 4 &&
+        (best == ctx->blocks.end() || b->bytes < best->bytes))
+      best = b;
+  DevBlock blk{nullptr, bytes};
+  if (best != ctx->blocks.end()) {
+    blk = *best;
+    ctx->blocks.erase(best);
+  } else {
+    cudaError_t e = cudaMalloc(&blk.p, bytes);
+    if (e == cudaErrorMemoryAllocation && !ctx->blocks.empty()) {
+      for (const DevBlock& b : ctx->blocks) cudaFree(b.p);
+      ctx->blocks.clear();
+      cudaGetLastError();
+      e = cudaMalloc(&blk.p, bytes);
+    }
+    if (e != cudaSuccess) return salf_cuda_fail(e, "cudaMalloc(scene)");
+  }
+  s->blocks.push_back(blk);
+  s->device_bytes += (int64_t)bytes;
+  *p = blk.p;
+  return SALF_OK;
+}
+
+// A scene's blocks go back to its context while the device is idle, the oldest
+// ones there to the device.
+static void keep_blocks(salf_ctx* ctx, const std::vector<DevBlock>& blocks) {
+  std::lock_guard<std::mutex> lk(ctx->blocks_mu);
+  size_t sum = 0;
+  ctx->blocks.insert(ctx->blocks.end(), blocks.begin(), blocks.end());
+  for (const DevBlock& b : ctx->blocks) sum += b.bytes;
+  while (sum > kBlocksKeep) {
+    sum -= ctx->blocks.front().bytes;
+    cudaFree(ctx->blocks.front().p);
+    ctx->blocks.erase(ctx->blocks.begin());
+  }
 }
 
 void salf_scene_hold_ctx(salf_scene* s, salf_ctx* ctx) {
@@ -102,6 +147,7 @@ extern "C" void salf_scene_destroy(salf_scene* s) {
   cudaSetDevice(s->device);
   cudaDeviceSynchronize();
   for (void* p : s->allocations) cudaFreeAsync(p, 0);  // the device is idle
+  if (s->ctx) keep_blocks(s->ctx, s->blocks);
   if (s->staging) cudaFree(s->staging);
   if (s->grads) cudaFree(s->grads);
   if (s->raster_vox) cudaFree(s->raster_vox);

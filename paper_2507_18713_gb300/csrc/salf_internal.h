@@ -171,9 +171,17 @@ struct LaunchParams {
 // ---------------------------------------------------------------- host side
 
 // Device memory of scenes and of their builds comes from a pool of the
-// context's own, which keeps up to kPoolKeep freed bytes for the next build
-// (cudaMalloc and cudaFree took more than half of a 1M-voxel rebuild).
-constexpr unsigned long long kPoolKeep = 1ull << 30;
+// context's own (cudaMalloc and cudaFree took more than half of a 1M-voxel
+// rebuild).  What callers get pointers to, records and voxel order, comes from
+// cudaMalloc, as pool memory can be neither exported (cudaIpcGetMemHandle) nor
+// read by peers; freed blocks of it are kept for the next scene (a 162 MB block:
+// 40 us to allocate, 103 to free).  The context keeps this much of each.
+constexpr unsigned long long kPoolKeep = 512ull << 20, kBlocksKeep = 512ull << 20;
+
+struct DevBlock {
+  void* p;
+  size_t bytes;
+};
 
 // Held by its creator until salf_destroy and by each of its scenes: calls on a
 // scene may take temporaries from the pool, which goes with the last holder.
@@ -181,6 +189,8 @@ struct salf_ctx {
   int device;
   cudaMemPool_t pool = nullptr;
   std::atomic<int> holders{1};
+  std::mutex blocks_mu;
+  std::vector<DevBlock> blocks;  // freed, oldest first
 };
 
 struct salf_scene {
@@ -193,7 +203,8 @@ struct salf_scene {
   double origin[3] = {0, 0, 0};
   double s0 = 0, sfin = 0;
   int64_t n_cells0 = 0, n_nodes = 0, device_bytes = 0;
-  std::vector<void*> allocations;  // every device buffer the scene owns
+  std::vector<void*> allocations;  // the scene's buffers from the pool
+  std::vector<DevBlock> blocks;    // and from cudaMalloc
   // library-owned FP32 gradient buffer (n x 32, input order; salf_scene_params)
   std::mutex grads_mu;
   float* grads = nullptr;
@@ -282,8 +293,10 @@ void salf_grid_shape(const int32_t dims[3], int mdim[3], int* p, int* q);
 // The skip boxes of s->dev from its occupancy words and tight box (D.mask0,
 // D.mdim0, D.mdim01, D.bmin, D.bmax, D.K set); asynchronous on `st`.
 salf_status salf_build_skip(salf_scene* s, int p, int q, cudaStream_t st);
-// A device buffer owned (and freed) by the scene.
+// A device buffer owned (and freed) by the scene, from its context's pool; and one
+// whose pointer callers get.
 salf_status salf_scene_dalloc(salf_scene* s, size_t bytes, void** p);
+salf_status salf_scene_block(salf_scene* s, size_t bytes, void** p);
 // Keep a copy of the build's voxel keys in the scene (for salf_scene_save).
 salf_status salf_scene_keep_keys(salf_scene* s, const salf_scene_desc* d);
 salf_status salf_prepare_request(const salf_scene* sc, const salf_sensor* sen,

@@ -56,9 +56,10 @@ salf_status dalloc(salf_scene* s, size_t bytes, void** p) {
 }
 
 template <class T>
-salf_status upload(salf_scene* s, const std::vector<T>& v, T** out) {
+salf_status upload(salf_scene* s, const std::vector<T>& v, T** out,
+                   salf_status (*alloc)(salf_scene*, size_t, void**) = dalloc) {
   void* p = nullptr;
-  salf_status st = dalloc(s, v.size() * sizeof(T), &p);
+  salf_status st = alloc(s, v.size() * sizeof(T), &p);
   if (st != SALF_OK) return st;
   if (!v.empty()) {
     cudaError_t e = cudaMemcpy(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
@@ -291,7 +292,7 @@ salf_status salf_build_scene_impl(salf_ctx* ctx, const salf_scene_desc* d, salf_
   if ((st = upload(s, nodes, &dnodes)) != SALF_OK) return st;
   std::vector<int32_t> ord = order;
   if (ord.empty()) ord.push_back(0);
-  if ((st = upload(s, ord, &dorder)) != SALF_OK) return st;
+  if ((st = upload(s, ord, &dorder, salf_scene_block)) != SALF_OK) return st;
   D.cells = dcells;
   D.nodes = dnodes;
   D.order = dorder;
@@ -313,7 +314,8 @@ salf_status salf_build_scene_impl(salf_ctx* ctx, const salf_scene_desc* d, salf_
   D.status = static_cast<int*>(status);
   void* params = nullptr;
   const size_t rec_bytes = d->dtype == SALF_F32 ? 128 : 64;
-  if ((st = dalloc(s, (size_t)std::max<int64_t>(n, 1) * rec_bytes, &params)) != SALF_OK) return st;
+  if ((st = salf_scene_block(s, (size_t)std::max<int64_t>(n, 1) * rec_bytes, &params)) != SALF_OK)
+    return st;
   D.params = params;
   for (int a = 0; a < 3; ++a) {
     D.origin[a] = d->origin[a];

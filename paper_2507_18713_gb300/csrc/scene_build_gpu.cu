@@ -389,9 +389,10 @@ salf_status salf_build_scene_gpu(salf_ctx* ctx, const salf_scene_desc* d, salf_s
   const size_t rec_bytes = d->dtype == SALF_F32 ? 128 : 64;
   if ((sst = alloc(nb0 * sizeof(uint4), &pmask0)) != SALF_OK ||
       (sst = alloc(nn * sizeof(int2), &pcells)) != SALF_OK ||
-      (sst = alloc(nn * sizeof(int), &pord)) != SALF_OK ||
+      (sst = salf_scene_block(s, nn * sizeof(int), &pord)) != SALF_OK ||
       (sst = alloc(nn * sizeof(int4), &pbox)) != SALF_OK ||
-      (sst = alloc(16, &pstatus)) != SALF_OK || (sst = alloc(nn * rec_bytes, &params)) != SALF_OK)
+      (sst = alloc(16, &pstatus)) != SALF_OK ||
+      (sst = salf_scene_block(s, nn * rec_bytes, &params)) != SALF_OK)
     return sst;
   uint4* mask0 = static_cast<uint4*>(pmask0);
   int2* cells = static_cast<int2*>(pcells);

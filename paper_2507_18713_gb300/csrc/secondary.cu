@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(256) k_secondary(const __grid_constant__ Secon
       p[k] = pair_add(Pair{r.Of[k], 0.f},
                       pair_mul(Pair{td, __fmaf_rn(ts, r.d[k], -td)}, S.isf2));
       float frac;
-      c[k] = r.Oi[k] + pair_floor(p[k], &frac);
+      c[k] = r.Oi[k] + pair_floor(p[k], p[k].hi, &frac);
       // (not a number, or beyond any grid: no hit point)
       inside = inside && fabsf(p[k].hi) < 1e9f && c[k] >= 0 && c[k] < S.Gf[k];
     }

@@ -43,7 +43,6 @@ __device__ __forceinline__ Pair pair_add(Pair a, Pair b) {
 
 __device__ __forceinline__ Pair pair_mul(Pair a, const float b[2]) {
   const float p = __fmul_rn(a.hi, b[0]);
-  if (fabsf(p) > 3.4e38f) return Pair{p, 0.f};  // beyond floats: no rounding error to follow
   const float e = __fmaf_rn(a.hi, b[0], -p);
   return two_sum(p, __fmaf_rn(a.hi, b[1], __fmaf_rn(a.lo, b[0], e)));
 }
@@ -54,11 +53,12 @@ __device__ __forceinline__ Pair pair_mul(Pair a, const float b[2]) {
 constexpr int kFarCell = 0x7f800000;
 
 // A pair as an int and a fraction in [0, 1] (1: less than 1 by under 2^-25).
-// Beyond kFarCell: there, and no fraction.
-__device__ __forceinline__ int pair_floor(Pair a, float* frac) {
-  if (fabsf(a.hi) >= (float)kFarCell) {
+// Where it is beyond kFarCell: there, and no fraction.  `about` is its value to
+// one float, which may be infinite (the pair is NaN then).
+__device__ __forceinline__ int pair_floor(Pair a, float about, float* frac) {
+  if (fabsf(about) >= (float)kFarCell) {
     *frac = 0.f;
-    return a.hi < 0.f ? -kFarCell : kFarCell;
+    return about < 0.f ? -kFarCell : kFarCell;
   }
   const float f = floorf(a.hi);
   const float r = __fadd_rn(__fsub_rn(a.hi, f), a.lo);
@@ -80,9 +80,8 @@ __device__ __forceinline__ void gen_ray(const ReqDev& Q, const DevScene& S, int 
     const float o[3] = {a.x, a.y, a.z};
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      const Pair g = pair_mul(pair_add(Pair{o[k], 0.f}, Pair{-S.origin2[k][0], -S.origin2[k][1]}),
-                              S.isf2);
-      r.Oi[k] = pair_floor(g, &r.Of[k]);
+      const Pair d = pair_add(Pair{o[k], 0.f}, Pair{-S.origin2[k][0], -S.origin2[k][1]});
+      r.Oi[k] = pair_floor(pair_mul(d, S.isf2), __fmul_rn(d.hi, S.isf2[0]), &r.Of[k]);
     }
     float dx = a.w, dy = b.x, dz = b.y;
     float nn = dx * dx + dy * dy + dz * dz;

@@ -68,10 +68,42 @@ extern "C" void salf_destroy(salf_ctx* ctx) {
   delete ctx;
 }
 
+// All that the context keeps for later goes back to the device.
+static void give_back(salf_ctx* ctx) {
+  std::lock_guard<std::mutex> lk(ctx->blocks_mu);
+  for (const DevBlock& b : ctx->blocks) cudaFree(b.p);
+  ctx->blocks.clear();
+  cudaStreamSynchronize(0);  // frees that have not run yet cannot be trimmed
+  cudaMemPoolTrimTo(ctx->pool, 0);
+  cudaGetLastError();  // the failed allocation's
+}
+
+cudaError_t salf_dev_malloc(salf_ctx* ctx, void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    give_back(ctx);
+    e = cudaMalloc(p, bytes);
+  }
+  if (e != cudaSuccess) *p = nullptr;
+  return e;
+}
+
+cudaError_t salf_pool_malloc(salf_ctx* ctx, void** p, size_t bytes, cudaStream_t st) {
+  cudaError_t e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, st);
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (e == cudaErrorMemoryAllocation && cudaStreamIsCapturing(st, &cap) == cudaSuccess &&
+      cap == cudaStreamCaptureStatusNone) {
+    give_back(ctx);
+    e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, st);
+  }
+  if (e != cudaSuccess) *p = nullptr;
+  return e;
+}
+
 salf_status salf_scene_block(salf_scene* s, size_t bytes, void** p) {
   salf_ctx* ctx = s->ctx;
   bytes = std::max<size_t>(bytes, 16);
-  std::lock_guard<std::mutex> lk(ctx->blocks_mu);
+  std::unique_lock<std::mutex> lk(ctx->blocks_mu);
   // the smallest kept block that holds it and is at most a quarter larger
   auto best = ctx->blocks.end();
   for (auto b = ctx->blocks.begin(); b != ctx->blocks.end(); ++b)
@@ -83,13 +115,8 @@ salf_status salf_scene_block(salf_scene* s, size_t bytes, void** p) {
     blk = *best;
     ctx->blocks.erase(best);
   } else {
-    cudaError_t e = cudaMalloc(&blk.p, bytes);
-    if (e == cudaErrorMemoryAllocation && !ctx->blocks.empty()) {
-      for (const DevBlock& b : ctx->blocks) cudaFree(b.p);
-      ctx->blocks.clear();
-      cudaGetLastError();
-      e = cudaMalloc(&blk.p, bytes);
-    }
+    lk.unlock();
+    const cudaError_t e = salf_dev_malloc(ctx, &blk.p, bytes);
     if (e != cudaSuccess) return salf_cuda_fail(e, "cudaMalloc(scene)");
   }
   s->blocks.push_back(blk);
@@ -119,11 +146,8 @@ void salf_scene_hold_ctx(salf_scene* s, salf_ctx* ctx) {
 }
 
 salf_status PoolBuf::get(salf_ctx* ctx, size_t bytes, cudaStream_t stream) {
-  const cudaError_t e = cudaMallocFromPoolAsync(&p, bytes ? bytes : 16, ctx->pool, stream);
-  if (e != cudaSuccess) {
-    p = nullptr;
-    return salf_cuda_fail(e, "cudaMallocFromPoolAsync");
-  }
+  const cudaError_t e = salf_pool_malloc(ctx, &p, bytes ? bytes : 16, stream);
+  if (e != cudaSuccess) return salf_cuda_fail(e, "cudaMallocFromPoolAsync");
   st = stream;
   return SALF_OK;
 }
@@ -197,7 +221,8 @@ extern "C" salf_status salf_scene_params(salf_scene* s, void** dev_params, void*
     if ((e = cudaSetDevice(s->device)) != cudaSuccess) return salf_cuda_fail(e, "cudaSetDevice");
     const size_t bytes = (size_t)(s->n > 0 ? s->n : 1) * SALF_RECORD_SCALARS * sizeof(float);
     float* g = nullptr;
-    if ((e = cudaMalloc(&g, bytes)) != cudaSuccess) return salf_cuda_fail(e, "cudaMalloc(grads)");
+    if ((e = salf_dev_malloc(s->ctx, reinterpret_cast<void**>(&g), bytes)) != cudaSuccess)
+      return salf_cuda_fail(e, "cudaMalloc(grads)");
     if ((e = cudaMemset(g, 0, bytes)) != cudaSuccess) {
       cudaFree(g);
       return salf_cuda_fail(e, "cudaMemset(grads)");
@@ -243,7 +268,7 @@ static salf_status ensure_staging(salf_scene* s, size_t bytes) {
     s->staging = nullptr;
     s->staging_bytes = 0;
   }
-  cudaError_t e = cudaMalloc(&s->staging, bytes);
+  cudaError_t e = salf_dev_malloc(s->ctx, &s->staging, bytes);
   if (e != cudaSuccess) {
     s->staging = nullptr;
     return salf_cuda_fail(e, "cudaMalloc(staging)");
@@ -992,7 +1017,7 @@ extern "C" salf_status salf_render_rays_actors(salf_scene* sc, const salf_actor*
     sc->actor_buf = nullptr;
     sc->actor_buf_bytes = 0;
     const size_t grow = bytes + bytes / 4;
-    if (cudaMalloc(&sc->actor_buf, grow) != cudaSuccess) {
+    if (salf_dev_malloc(sc->ctx, &sc->actor_buf, grow) != cudaSuccess) {
       cudaGetLastError();
       g_err = "salf_render_rays_actors: out of device memory";
       return SALF_ERR_OOM;
@@ -1133,7 +1158,7 @@ extern "C" salf_status salf_render_backward_actors(
     sc->actor_buf = nullptr;
     sc->actor_buf_bytes = 0;
     const size_t grow = bytes + bytes / 4;
-    if (cudaMalloc(&sc->actor_buf, grow) != cudaSuccess) {
+    if (salf_dev_malloc(sc->ctx, &sc->actor_buf, grow) != cudaSuccess) {
       cudaGetLastError();
       g_err = "salf_render_backward_actors: out of device memory";
       return SALF_ERR_OOM;

@@ -510,7 +510,7 @@ salf_status salf_raster_run(salf_scene* sc, const ReqDev& r, double fx, double f
     if (sc->raster_vox) cudaFree(sc->raster_vox);
     sc->raster_vox = nullptr;
     sc->raster_vox_bytes = 0;
-    if (cudaMalloc(&sc->raster_vox, need_vox) != cudaSuccess) {
+    if (salf_dev_malloc(sc->ctx, &sc->raster_vox, need_vox) != cudaSuccess) {
       cudaGetLastError();
       salf_set_error("salf_render_raster: out of device memory (voxel workspace)");
       return SALF_ERR_OOM;
@@ -592,7 +592,7 @@ salf_status salf_raster_run(salf_scene* sc, const ReqDev& r, double fx, double f
     sc->raster_pairs = nullptr;
     sc->raster_pairs_bytes = 0;
     const size_t grow = need_pairs + need_pairs / 4;
-    if (cudaMalloc(&sc->raster_pairs, grow) != cudaSuccess) {
+    if (salf_dev_malloc(sc->ctx, &sc->raster_pairs, grow) != cudaSuccess) {
       cudaGetLastError();
       salf_set_error("salf_render_raster: out of device memory (tile lists)");
       return SALF_ERR_OOM;

@@ -349,7 +349,7 @@ extern "C" salf_status salf_scene_refine_plan(salf_scene* sc, const float* grads
     if (sc->refine_ws) cudaFree(sc->refine_ws);
     sc->refine_ws = nullptr;
     sc->refine_ws_bytes = 0;
-    if (cudaMalloc(&sc->refine_ws, need) != cudaSuccess) {
+    if (salf_dev_malloc(sc->ctx, &sc->refine_ws, need) != cudaSuccess) {
       cudaGetLastError();
       salf_set_error("salf_scene_refine_plan: out of device memory");
       return SALF_ERR_OOM;

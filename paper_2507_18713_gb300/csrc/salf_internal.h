@@ -277,6 +277,10 @@ struct SalfRange {
 
 // Implemented in the .cu / .cpp files of the library.
 void salf_set_error(const std::string& msg);
+// cudaMalloc / an allocation from the context's pool; where the device has no room,
+// the context gives back what it keeps before they are tried again.
+cudaError_t salf_dev_malloc(salf_ctx* ctx, void** p, size_t bytes);
+cudaError_t salf_pool_malloc(salf_ctx* ctx, void** p, size_t bytes, cudaStream_t st);
 // The scene holds the context from here on (salf_scene_destroy lets go of it).
 void salf_scene_hold_ctx(salf_scene* s, salf_ctx* ctx);
 salf_status salf_cuda_fail(cudaError_t e, const char* what);

@@ -42,9 +42,8 @@ struct Scope {  // frees a half-built scene on error
 
 salf_status dalloc(salf_scene* s, size_t bytes, void** p) {
   if (bytes == 0) bytes = 16;
-  cudaError_t e = cudaMallocFromPoolAsync(p, bytes, s->ctx->pool, 0);
+  cudaError_t e = salf_pool_malloc(s->ctx, p, bytes, 0);
   if (e != cudaSuccess) {
-    *p = nullptr;
     salf_set_error(std::string("device allocation (") + std::to_string(bytes) + ") failed: " +
                    cudaGetErrorString(e));
     cudaGetLastError();
@@ -348,7 +347,7 @@ salf_status salf_build_scene_impl(salf_ctx* ctx, const salf_scene_desc* d, salf_
     const float* src = d->params;
     void* tmp = nullptr;
     if (!d->params_on_device) {
-      if ((ce = cudaMalloc(&tmp, (size_t)n * 128)) != cudaSuccess) {
+      if ((ce = salf_dev_malloc(ctx, &tmp, (size_t)n * 128)) != cudaSuccess) {
         cudaGetLastError();
         salf_set_error("cudaMalloc(param staging) failed");
         return ce == cudaErrorMemoryAllocation ? SALF_ERR_OOM : SALF_ERR_CUDA;

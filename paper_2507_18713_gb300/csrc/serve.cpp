@@ -302,7 +302,7 @@ extern "C" salf_status salf_serve_create(salf_scene* scene, size_t budget, int32
   salf_server* s = new salf_server();
   s->scene = scene;
   budget = align256(budget);
-  e = cudaMalloc(reinterpret_cast<void**>(&s->arena_base), budget);
+  e = salf_dev_malloc(scene->ctx, reinterpret_cast<void**>(&s->arena_base), budget);
   if (e != cudaSuccess) {
     delete s;
     return salf_cuda_fail(e, "cudaMalloc(serve arena)");

@@ -74,3 +74,39 @@ def test_blocks_are_taken_again(salf):
     del ctx, g, held, h
     torch.cuda.synchronize()
     assert free0 - torch.cuda.mem_get_info()[0] <= 64 << 20
+
+
+def test_kept_memory_is_given_back(salf):
+    """What a context keeps for its next scenes is there for the library's other
+    allocations: on a full device, servers' arenas take it all."""
+    ctx = salf.Context(0)
+    sc = synth.random_multilevel_scene(seed=3, max_level=0, dims=(140, 140, 140), p_occ=0.9)
+    level, ijk = torch.from_numpy(sc.level).cuda(), torch.from_numpy(sc.ijk).cuda()
+    params = torch.from_numpy(np.asarray(sc.params, np.float32)).cuda()
+    part = lambda n: salf.Scene(salf.VoxelSet(sc.origin, sc.s0, sc.dims, 0, level[:n], ijk[:n],
+                                              params[:n], "exp"), ctx=ctx)
+    small = part(50000)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free0 = torch.cuda.mem_get_info()[0]
+    part(sc.n).close()  # leaves some 300 MB of records with the context, and pool memory
+    free1 = torch.cuda.mem_get_info()[0]
+    assert free0 - free1 > 300 << 20
+    room, arena = 48 << 20, 32 << 20
+    fill = torch.empty(free1 - room, dtype=torch.uint8, device="cuda")
+    servers = []
+    try:
+        for _ in range(64):
+            try:
+                servers.append(salf.Server(small, arena, n_streams=1))
+            except salf.SalfError as e:
+                assert e.status == 2  # out of memory
+                break
+    finally:
+        taken = len(servers) * arena
+        for s in servers:
+            s.close()
+        del fill
+        torch.cuda.empty_cache()
+    assert taken >= free0 - free1 + room - 3 * arena
+    small.close()

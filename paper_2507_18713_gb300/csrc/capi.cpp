@@ -502,10 +502,12 @@ salf_status salf_prepare_request(const salf_scene* sc, const salf_sensor* s,
 // 4 / 8 spans, us): 2M-voxel driving scene (side 1000) 1024x32 180 / 124 / 105,
 // 1024x64 231 / 180 / 140, 1024x128 236 / 177 / 179, 2400x128 257 / 236 / 392,
 // 4096x128 268 / 376 / 640; 200k voxels (side 316) 1024x32 89 / 77 / 73, 1024x64
-// 96 / 101 / 108, 2048x128 102 / 153 / 259.  Small camera frames would gain too (128x96:
-// 251 / 148 / 118), but cameras walk whole rays so that ray-cast and rasterised
-// frames stay equal bit for bit.  The choice is the sensor's alone: batches give
-// the outputs of lone calls.
+// 96 / 101 / 108, 2048x128 102 / 153 / 259.  (The lines, straight in the side, miss the
+// best of these in one place: 1024x64 on 200k voxels takes 4 spans, 5% slower than
+// whole rays.)  Small camera frames would gain too (128x96: 251 / 148 / 118), but
+// cameras walk whole rays so that ray-cast and rasterised
+// frames stay equal bit for bit.  The choice depends on the sensor and the scene,
+// never on the batch: batches give the outputs of lone calls.
 int salf_auto_segments(const salf_scene* sc, const salf_sensor* s) {
   if (s->kind != SALF_LIDAR_SPIN) return 1;
   int64_t side = 1;

@@ -288,9 +288,9 @@ __global__ void __launch_bounds__(kRasterThreads, SALF_RASTER_MIN_BLOCKS) k_rast
   // this warp's pixels: 8 columns x 4 rows (16 x 2 meet a fifth more voxels: 4K frame
   // 864 us against 842)
   const int warp = threadIdx.x >> 5;
-  const int strip_u0 = (tile % RP.tiles_x) * kTile + 8 * (warp & 1), strip_u1 = strip_u0 + 7;
-  const int strip_v0 = (tile / RP.tiles_x) * kTile + 4 * (warp >> 1), strip_v1 = strip_v0 + 3;
-  const int u = strip_u0 + (lane & 7), v = strip_v0 + (lane >> 3);
+  const int warp_u0 = (tile % RP.tiles_x) * kTile + 8 * (warp & 1), warp_u1 = warp_u0 + 7;
+  const int warp_v0 = (tile / RP.tiles_x) * kTile + 4 * (warp >> 1), warp_v1 = warp_v0 + 3;
+  const int u = warp_u0 + (lane & 7), v = warp_v0 + (lane >> 3);
   const bool in_img = u < Q.W && v < Q.H;
   const int ray = v * Q.W + u;
 
@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(kRasterThreads, SALF_RASTER_MIN_BLOCKS) k_rast
     const int n = (int)min((unsigned)kChunk, rg.y - c0);
     if (c0 != rg.x) fetch(c0, n);  // the previous chunk is no longer read (end of the loop)
     store(n);
-    // voxels whose pixel rectangle meets this warp's 16 x 2 pixel strip
+    // voxels whose pixel rectangle meets this warp's 8 x 4 pixels
     unsigned sel[kChunk / 32];
 #pragma unroll
     for (int q = 0; q < kChunk / 32; ++q) {
@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(kRasterThreads, SALF_RASTER_MIN_BLOCKS) k_rast
       bool meet = false;
       if (j < n) {
         const int4 pr = s_prect[j];
-        meet = pr.x <= strip_u1 && pr.y >= strip_u0 && pr.z <= strip_v1 && pr.w >= strip_v0;
+        meet = pr.x <= warp_u1 && pr.y >= warp_u0 && pr.z <= warp_v1 && pr.w >= warp_v0;
       }
       sel[q] = __ballot_sync(0xffffffffu, meet);
     }
@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(kRasterThreads, SALF_RASTER_MIN_BLOCKS) k_rast
       *tin_out = tin;
       *tout_out = fminf(fminf(fminf(tx[0], tx[1]), tx[2]), w.t1);
     };
-    // phase 1: which of the strip's voxels this pixel's ray crosses
+    // phase 1: which of the warp's voxels this pixel's ray crosses
     unsigned hits[kChunk / 32];
 #pragma unroll
     for (int q = 0; q < kChunk / 32; ++q) {

@@ -350,7 +350,7 @@ __device__ __forceinline__ void actor_walk(const ActorDev& A, const Ray& r, Walk
   for (int a = 0; a < 3; ++a) {
     const float g = (oc[a] - A.origin[a]) * A.inv_sfin;
     const float f = floorf(g);
-    ra.Oi[a] = min(max((int)f, -kFarCell), kFarCell);
+    ra.Oi[a] = (int)fminf(fmaxf(f, -(float)kFarCell), (float)kFarCell);
     ra.Of[a] = g - f;
     ra.d[a] = dc[a];
   }

@@ -102,7 +102,11 @@ cudaError_t salf_pool_malloc(salf_ctx* ctx, void** p, size_t bytes, cudaStream_t
 
 salf_status salf_scene_block(salf_scene* s, size_t bytes, void** p) {
   salf_ctx* ctx = s->ctx;
-  bytes = std::max<size_t>(bytes, 16);
+  // sizes in steps of a sixteenth of their power of two: the next scene of about
+  // this size takes the same block
+  size_t step = 16;
+  while (step * 32 <= bytes) step *= 2;
+  bytes = std::max<size_t>(bytes + step - 1, 16) / step * step;
   std::unique_lock<std::mutex> lk(ctx->blocks_mu);
   // the smallest kept block that holds it and is at most a quarter larger
   auto best = ctx->blocks.end();

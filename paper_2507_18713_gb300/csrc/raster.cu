@@ -10,7 +10,7 @@
 //  4. stable LSD radix sort of the pairs, 8 bits per pass;
 //  5. k_tile_ranges: each tile's slice of the sorted pairs;
 //  6. k_raster: one 256-thread block per tile, one thread per pixel; the
-//     tile's voxels are staged kChunk at a time in shared memory (records raw,
+//     tile's voxels are staged a chunk at a time in shared memory (records raw,
 //     boxes as plane offsets) and composited front to back with early
 //     termination, with the ray kernel's ray set-up, slab test and field code.
 //
@@ -37,20 +37,24 @@ using namespace salf_sort;
 
 namespace {
 
-// Resident tile blocks per SM the register budget must allow: 5 x 8 warps in 48
-// registers; spills cost less than the barrier waits that they hide (4K frame: 3
-// blocks 976 us, 4 890, 5 867; 5 with 64-voxel chunks 831, 6 839).
-#ifndef SALF_RASTER_MIN_BLOCKS
-#define SALF_RASTER_MIN_BLOCKS 5
-#endif
-
 constexpr int kTile = 16;          // tile edge in pixels
 constexpr int kRasterThreads = kTile * kTile;
-#ifndef SALF_RASTER_CHUNK
-#define SALF_RASTER_CHUNK 64
-#endif
-constexpr int kChunk = SALF_RASTER_CHUNK;  // voxels staged in shared memory at a time
-static_assert(kChunk <= kRasterThreads, "one box per thread");
+
+// k_raster's variants: resident blocks per SM that the register budget must allow,
+// and voxels staged in shared memory at a time (at most one box per thread).  Large
+// frames have tiles enough to hide the barrier waits: 5 blocks in 48 registers,
+// whose spills cost less than the waits, with small chunks.  Small frames are
+// bound by their longest tile lists, walked chunk by chunk: 3 blocks in 80
+// registers, and fewer, larger chunks.  Measured (us a frame, 5 x 64 / 3 x 128; driving
+// scenes of 2M, 1M and 300k voxels, F32):
+//   480x270   (510 tiles)   2119 / 1739   1134 / 915   420 / 348
+//   960x540   (2040)        1042 / 854     674 / 566   296 / 258
+//   1920x1080 (8160)         614 / 530     429 / 380   256 / 239
+//   2560x1440 (14400)        593 / 580     417 / 451   295 / 318
+//   3840x2160 (32400)        811 / 905     675 / 738   489 / 539
+constexpr int kSmallFrameTiles = 10000;
+constexpr int kBlocksSmall = 3, kChunkSmall = 128;
+constexpr int kBlocksLarge = 5, kChunkLarge = 64;
 
 struct ProjParams {
   DevScene S;
@@ -272,8 +276,9 @@ struct RasterParams {
   int tiles_x;
 };
 
-template <int DT, int MODE, bool DUMP>
-__global__ void __launch_bounds__(kRasterThreads, SALF_RASTER_MIN_BLOCKS) k_raster(const __grid_constant__ RasterParams RP) {
+template <int DT, int MODE, bool DUMP, int MINB, int kChunk>
+__global__ void __launch_bounds__(kRasterThreads, MINB) k_raster(const __grid_constant__ RasterParams RP) {
+  static_assert(kChunk <= kRasterThreads, "one box per thread");
   constexpr int RQ = RecordLayout<DT>::kChunks;
   constexpr int RS = RQ + 1;  // padded record stride: lanes reading different records hit different banks
   __shared__ float4 s_rec[kChunk * RS];
@@ -441,13 +446,21 @@ __global__ void __launch_bounds__(kRasterThreads, SALF_RASTER_MIN_BLOCKS) k_rast
   }
 }
 
+template <int DT, int MODE, int MINB, int CHUNK>
+void launch_raster_as(const RasterParams& RP, int ntiles, bool dump, cudaStream_t st) {
+  if (dump)
+    k_raster<DT, MODE, true, MINB, CHUNK><<<ntiles, kRasterThreads, 0, st>>>(RP);
+  else
+    k_raster<DT, MODE, false, MINB, CHUNK><<<ntiles, kRasterThreads, 0, st>>>(RP);
+}
+
 template <int DT, int MODE>
 void launch_raster(const RasterParams& RP, int ntiles, bool dump, cudaStream_t st) {
   if (ntiles <= 0) return;
-  if (dump)
-    k_raster<DT, MODE, true><<<ntiles, kRasterThreads, 0, st>>>(RP);
+  if (ntiles <= kSmallFrameTiles)
+    launch_raster_as<DT, MODE, kBlocksSmall, kChunkSmall>(RP, ntiles, dump, st);
   else
-    k_raster<DT, MODE, false><<<ntiles, kRasterThreads, 0, st>>>(RP);
+    launch_raster_as<DT, MODE, kBlocksLarge, kChunkLarge>(RP, ntiles, dump, st);
 }
 
 int bit_width(unsigned long long x) {

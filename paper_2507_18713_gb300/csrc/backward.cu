@@ -16,23 +16,34 @@
 // (T, the suffix sums and dL/dtau need it) and queue the hit's coefficients
 // in a per-warp ring in shared memory; whenever 32 are queued, the whole warp
 // builds their 32-scalar gradient rows and adds them to the caller's
-// input-order FP32 buffer with 16-byte vector atomics.  Where 8 or more rows of
-// a batch are of one voxel, they are staged in shared memory and summed first.
+// input-order FP32 buffer with 16-byte vector atomics.  Where 4 or more rows of
+// a batch are of one voxel, they are staged in shared memory and summed first,
+// so that a buffer's scalar is rounded once per batch, not once per row.
 //
-// Bound by instruction issue (57% of slots, 20 of 32 lanes active in the walk).
-// Of a training step of 8 views of 960x640 (2720 us) the sums took 300 us and
-// the atomics 27: with staging only for groups of 8 or more, and those split
-// over 8 to 32 lanes instead of 8, in the ring's own slots, the step takes
-// 2620 us and a LiDAR fit of 64x1024 470 (before: 2726 and 481).  Groups of
-// fewer than 10 or 12 by atomics: 2664 or more; all of them: 3473.
+// Bound by instruction issue (50% of slots, one 960x640 view) and the waits for
+// shared memory and records.  The sums run on the whole warp at once, whatever its
+// groups: with barriers inside each group the groups took turns.  Adjoint of 8
+// views of 960x640 on 1M voxels (BF16; SDF in F32; a LiDAR of 64x1024 on it), us:
+//   groups of 4 or more, one sum a batch   1446   1769   297
+//   groups of 3 or more; of 2 or more      1489   1808;  1517   1840
+//   groups of 6 or more                    1440   1785
+// Without the split into parts the long groups' loops take 1763; with up to 8
+// parts instead of 4 it is 1610 (registers).  Each part with atomics of its own
+// took 1425 / 1779 / 326, but 2 to 8 roundings per batch: the run-to-run noise of
+// gradients doubled, and tripled where voxels are large on the screen.
 #include "traverse.cuh"
 
-// warps per block and resident blocks per SM asked of the compiler
+// warps per block
 #ifndef SALF_BWD_WARPS
 #define SALF_BWD_WARPS 4
 #endif
-#ifndef SALF_BWD_MIN_BLOCKS
-#define SALF_BWD_MIN_BLOCKS 4  // 16 warps per SM: training step 2621 us, LiDAR fit 466; 5: 2623, 466
+// Resident blocks per SM: static pinholes 5 (94 to 96 registers; 4: 1557 us for the 8
+// views), the rest 4 (114; 5: LiDAR 332 us instead of 307, with spills).
+#ifndef SALF_BWD_BLOCKS_LEAN
+#define SALF_BWD_BLOCKS_LEAN 5
+#endif
+#ifndef SALF_BWD_BLOCKS
+#define SALF_BWD_BLOCKS 4
 #endif
 
 using namespace salf;
@@ -42,7 +53,8 @@ using namespace salf;
 // and no intensity or raydrop terms are compiled in (8-camera training
 // adjoint measured 1.5% faster).
 template <int DT, int MODE, bool LEAN>
-__global__ void __launch_bounds__(32 * SALF_BWD_WARPS, SALF_BWD_MIN_BLOCKS)
+__global__ void __launch_bounds__(32 * SALF_BWD_WARPS,
+                                  LEAN ? SALF_BWD_BLOCKS_LEAN : SALF_BWD_BLOCKS)
     k_backward(const __grid_constant__ LaunchParams P) {
   // see next_hit: LiDAR fit 464 -> 443 us, 2400x128 on 1.5M voxels 721 -> 686 (SDF 823 ->
   // 783); training step (cameras) 2640 -> 2615, but for SDF fields 4126 -> 4279
@@ -117,60 +129,84 @@ __global__ void __launch_bounds__(32 * SALF_BWD_WARPS, SALF_BWD_MIN_BLOCKS)
   // gradient rows of n queued hits (n <= 32), summed per voxel, added to d_params
   auto flush = [&](int n) {
     const bool act = lane < n;
-    int key = 0;
-    float4 gr[8];
-    if (act) {
-      const float4* it = queue + ((head + lane) & (QN - 1)) * QW;
-      const float4 i0 = it[0], i1 = it[1], i2 = it[2], i3 = it[3];
-      key = __float_as_int(i0.x);
-      const float x0 = i0.y, x1 = i0.z, x2 = i0.w;
-      const float g1 = i3.x, g2 = i3.y, g3 = i3.z;  // gamma_0 is a constant
-      const float di = want_int ? i1.w : 0.f, dr = want_drop ? i2.w : 0.f;
-      gr[0] = make_float4(i1.x * x0, i1.x * x1, i1.x * x2, i1.x);
-      gr[1] = make_float4(i2.x * x0, i2.x * x1, i2.x * x2, i2.y * x0);
-      gr[2] = make_float4(i2.y * x1, i2.y * x2, i2.z * x0, i2.z * x1);
-      gr[3] = make_float4(i2.z * x2, i2.x * kSH0, i2.x * g1, i2.x * g2);
-      gr[4] = make_float4(i2.x * g3, i2.y * kSH0, i2.y * g1, i2.y * g2);
-      gr[5] = make_float4(i2.y * g3, i2.z * kSH0, i2.z * g1, i2.z * g2);
-      gr[6] = make_float4(i2.z * g3, MODE == SALF_FIELD_EXP ? 0.f : i1.y,
-                          MODE == SALF_FIELD_EXP ? 0.f : i1.z, di * x0);
-      gr[7] = make_float4(di * x1, di * x2, di, dr);
+    // (a lane without a hit reads its slot of the ring all the same, and is a group of
+    // its own)
+    float4* slot = queue + ((head + lane) & (QN - 1)) * QW;
+    const float4 i0 = slot[0], i1 = slot[1], i2 = slot[2], i3 = slot[3];
+    const int key = act ? __float_as_int(i0.x) : -1 - lane;
+    const float x0 = i0.y, x1 = i0.z, x2 = i0.w;
+    const float di = want_int ? i1.w : 0.f, dr = want_drop ? i2.w : 0.f;
+    // chunk q of the hit's gradient row (gamma_0 is a constant)
+    auto chunk = [&](int q) {
+      switch (q) {
+        case 0: return make_float4(i1.x * x0, i1.x * x1, i1.x * x2, i1.x);
+        case 1: return make_float4(i2.x * x0, i2.x * x1, i2.x * x2, i2.y * x0);
+        case 2: return make_float4(i2.y * x1, i2.y * x2, i2.z * x0, i2.z * x1);
+        case 3: return make_float4(i2.z * x2, i2.x * kSH0, i2.x * i3.x, i2.x * i3.y);
+        case 4: return make_float4(i2.x * i3.z, i2.y * kSH0, i2.y * i3.x, i2.y * i3.y);
+        case 5: return make_float4(i2.y * i3.z, i2.z * kSH0, i2.z * i3.x, i2.z * i3.y);
+        case 6:
+          return make_float4(i2.z * i3.z, MODE == SALF_FIELD_EXP ? 0.f : i1.y,
+                             MODE == SALF_FIELD_EXP ? 0.f : i1.z, di * x0);
+        default: return make_float4(di * x1, di * x2, di, dr);
+      }
+    };
+    float4* dst = reinterpret_cast<float4*>(Q.d_params) + (size_t)key * 8;
+    const unsigned peers = __match_any_sync(0xffffffffu, key);
+    const int gn = __popc(peers);
+    const bool staged = gn >= 4;
+    if (act && !staged) {  // few rows of this voxel: their atomics cost less than staging
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (q < nq) atomicAdd(dst + q, chunk(q));
     }
-    const unsigned act_lanes = __ballot_sync(0xffffffffu, act);
-    if (act) {
-      const unsigned peers = __match_any_sync(act_lanes, key);
-      float4* dst = reinterpret_cast<float4*>(Q.d_params) + (size_t)key * 8;
-      const int gn = __popc(peers);
-      if (gn < 8) {  // few rows of this voxel: their atomics cost less than staging
+    if (__any_sync(0xffffffffu, staged)) {
+      // A group's rows in parts by lane, as the bits of `every` pick them: 1 (4-7 rows), 2
+      // (8-15) or 4; four lanes to a part, each summing one of its chunks.
+      const int rank = __popc(peers & ((1u << lane) - 1u));
+      const int parts = gn >= 16 ? 4 : gn >= 8 ? 2 : 1, part = rank >> 2, c = rank & 3;
+      const unsigned every = parts == 4 ? 0x11111111u : parts == 2 ? 0x55555555u : 0xffffffffu;
+      const unsigned mine = staged && part < parts ? peers & (every << part) : 0u;
+      // the lanes 4 and 8 ranks up hold the sums of the next part and of the one after
+      unsigned up = peers & ~((2u << lane) - 1u);
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-          if (q < nq) atomicAdd(dst + q, gr[q]);
-      } else {
-        // 8-15 rows in 2 parts, 16-31 in 4, 32 in 8, by lane: four lanes to a part,
-        // each summing one of its chunks (in 1, 2 and 4 parts: 2711 us, in 1: 2866)
-        const int rank = __popc(peers & ((1u << lane) - 1u));
-        const int parts = gn >= 32 ? 8 : gn >= 16 ? 4 : 2, part = rank >> 2, c = rank & 3;
-        const unsigned every = parts == 8 ? 0x01010101u : parts == 4 ? 0x11111111u : 0x55555555u;
-        const unsigned mine = part < parts ? peers & (every << part) : 0u;
-        // staged in the rows' own slots of the ring (each lane has read its hit), four
-        // chunks at a time
-        float4* slot = queue + ((head + lane) & (QN - 1)) * QW;
+      for (int k = 0; k < 3; ++k) up &= up - 1u;
+      const int up4 = (__ffs(up) - 1) & 31;
 #pragma unroll
-        for (int q0 = 0; q0 < 8; q0 += 4) {
+      for (int k = 0; k < 4; ++k) up &= up - 1u;
+      const int up8 = (__ffs(up) - 1) & 31;
+      const bool any2 = __any_sync(0xffffffffu, parts >= 2), any4 = __any_sync(0xffffffffu, parts == 4);
+      // staged in the rows' own slots of the ring (each lane has read its hit), four
+      // chunks at a time
 #pragma unroll
-          for (int q = 0; q < 4; ++q) slot[q] = gr[q0 + q];
-          __syncwarp(peers);
-          float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-          for (unsigned m = mine; m; m &= m - 1u) {
-            const float4 r2 = queue[((head + __ffs(m) - 1) & (QN - 1)) * QW + c];
-            sum.x += r2.x;
-            sum.y += r2.y;
-            sum.z += r2.z;
-            sum.w += r2.w;
-          }
-          if (mine && q0 + c < nq) atomicAdd(dst + q0 + c, sum);
-          __syncwarp(peers);
+      for (int q0 = 0; q0 < 8; q0 += 4) {
+        if (staged) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) slot[q] = chunk(q0 + q);
         }
+        __syncwarp();
+        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (unsigned m = mine; m; m &= m - 1u) {
+          const float4 r2 = queue[((head + __ffs(m) - 1) & (QN - 1)) * QW + c];
+          sum.x += r2.x;
+          sum.y += r2.y;
+          sum.z += r2.z;
+          sum.w += r2.w;
+        }
+        auto fold = [&](int from, bool take) {
+          const float x = __shfl_sync(0xffffffffu, sum.x, from),
+                      y = __shfl_sync(0xffffffffu, sum.y, from),
+                      z = __shfl_sync(0xffffffffu, sum.z, from),
+                      t = __shfl_sync(0xffffffffu, sum.w, from);
+          sum.x += take ? x : 0.f;
+          sum.y += take ? y : 0.f;
+          sum.z += take ? z : 0.f;
+          sum.w += take ? t : 0.f;
+        };
+        if (any4) fold(up8, parts == 4);  // parts 0 and 1 take 2 and 3
+        if (any2) fold(up4, parts >= 2);  // part 0 takes 1
+        if (staged && part == 0 && q0 + c < nq) atomicAdd(dst + q0 + c, sum);
+        __syncwarp();
       }
     }
     head += n;

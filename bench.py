@@ -746,7 +746,10 @@ def main():
                               kernel="k_raster<F32,EXP> (whole pipeline timed)" if raster
                               else "k_forward<F32,EXP>",
                               note="bytes = visits x record scalars read + outputs per ray; "
-                                   "visits counted by the kernel",
+                                   "visits counted by the kernel.  Most of these reads are "
+                                   "served by L1 and L2 (traffic = DRAM bytes of the launch): "
+                                   "the kernel is bound by issue (issue_frac), and frac can "
+                                   "pass 1",
                               l2=dict(peak_gbs=l2_peak,
                                       bytes_per_launch=l2_bytes,
                                       achieved_gbs=(l2_bytes / (avg * 1e-3) / 1e9

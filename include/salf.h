@@ -156,8 +156,11 @@ typedef struct {
  * consecutive spans); a part in which the ray actually stopped is walked
  * again from the transmittance in front of it, so the outputs are those of
  * the whole-ray walk up to rounding.  It shortens the longest rays' serial
- * latency (LiDAR beams near the horizon).  0 = the library's choice per
- * sensor kind.  Renders that record visits, ray dumps, step counts or alpha
+ * latency (LiDAR beams near the horizon).  0 = the library's choice: whole
+ * rays, and for spinning LiDARs 8 parts up to 128 rays per level-0 cell of the
+ * longest side of the voxels' box (at most 81920 rays), 4 up to 320 (at most
+ * 327680), whole rays beyond; a sensor's choice is the same in any batch.
+ * Renders that record visits, ray dumps, step counts or alpha
  * maxima, rasterised and actor renders and the backward pass walk whole rays.
  */
 typedef struct {
@@ -181,7 +184,8 @@ typedef struct {
  *   visit_count, visits: see salf_render_opts.visits_cap
  *   ray_dump  R x 8 (debugging aid): the generated ray as (ox, oy, oz, dx, dy,
  *             dz, time, valid) in world coordinates
- *   steps     R (debugging aid): structure leaves the traversal stepped through
+ *   steps     R (debugging aid): structure steps of the traversal (voxels, cells
+ *             and skip boxes left)
  *   raydrop   R: sum_i T_i alpha_i sigmoid(rho_i) + T_end, the probability that
  *             the LiDAR return is dropped (a ray that leaves the scene returns
  *             nothing); Sec. V-C and Table III name raydrop without a form.
@@ -239,11 +243,28 @@ void salf_destroy(salf_ctx* ctx);
 
 /*
  * Build a scene (Sec. III-A representation, Sec. III-B acceleration
- * structure).  Voxels are sorted in Morton order of their min corner, checked
- * for overlaps, and indexed by an occupancy pyramid of 64-bit masks over 4^3
- * blocks (with rank offsets into the level-0 cell table) plus 8-way
- * subdivision nodes below level 0.  Synchronous.  Errors: INVALID (sizes,
- * ranges, SDF a or b <= 0), OVERLAP, OOM, CUDA.
+ * structure).  Voxels are sorted block by block (4^3 level-0 cells; Morton
+ * order of cells and of min corners inside), checked for overlaps, and indexed
+ * by one 64-bit occupancy mask per block (with rank offsets into the level-0
+ * cell table) plus 8-way subdivision nodes below level 0.  Empty space is
+ * indexed by skip boxes: the voxels' tight box is cut into bricks of 4x4x1
+ * level-0 cells (larger ones in grids of more than 2^28), and an empty brick
+ * holds, for each of the 8 direction octants, the size of an empty box that a
+ * ray leaves in one step.  Synchronous.
+ *
+ * Device memory of a scene: 16 B per 4^3 block of the grid, 16 B per brick of
+ * the tight box, 8 B per occupied level-0 cell (per voxel if built from device
+ * keys), 32 B per node, 33 B per voxel, and its record (128 B FP32, 64 B BF16);
+ * salf_scene_info.device_bytes has the sum.  A build needs in passing 208 B per
+ * column of bricks and 64 layers (21 GB for voxels that span 40000 x 40000 x 4
+ * cells), and from device keys 26 to 42 B per voxel and 24 B per block, from
+ * host arrays 128 B per voxel.
+ * Records and voxel order are cudaMalloc memory, the rest is from a memory pool
+ * of the context.  A context keeps up to 512 MB of each for its next scenes; an
+ * allocation of the library's that finds no room takes them back first, one of
+ * the caller's does not: salf_destroy gives them back.
+ *
+ * Errors: INVALID (sizes, ranges, SDF a or b <= 0), OVERLAP, OOM, CUDA.
  */
 salf_status salf_build_scene(salf_ctx* ctx, const salf_scene_desc* desc, salf_scene** out);
 void salf_scene_destroy(salf_scene* scene);

@@ -20,7 +20,7 @@
 // a batch are of one voxel, they are staged in shared memory and summed first,
 // so that a buffer's scalar is rounded once per batch, not once per row.
 //
-// Bound by instruction issue (50% of slots, one 960x640 view) and the waits for
+// Bound by instruction issue (59% of slots, 24 of 32 lanes) and the waits for
 // shared memory and records.  The sums run on the whole warp at once, whatever its
 // groups: with barriers inside each group the groups took turns.  Adjoint of 8
 // views of 960x640 on 1M voxels (BF16; SDF in F32; a LiDAR of 64x1024 on it), us:

@@ -260,9 +260,10 @@ void salf_destroy(salf_ctx* ctx);
  * cells), and from device keys 26 to 42 B per voxel and 24 B per block, from
  * host arrays 128 B per voxel.
  * Records and voxel order are cudaMalloc memory, the rest is from a memory pool
- * of the context.  A context keeps up to 512 MB of each for its next scenes; an
- * allocation of the library's that finds no room takes them back first, one of
- * the caller's does not: salf_destroy gives them back.
+ * of the context.  A context keeps freed memory for its next scenes: up to 512 MB
+ * of the former, and of the pool's while it holds less than 1 GB in all.  An
+ * allocation of the library's that finds no room takes it back first, one of
+ * the caller's does not; salf_destroy gives it back.
  *
  * Errors: INVALID (sizes, ranges, SDF a or b <= 0), OVERLAP, OOM, CUDA.
  */

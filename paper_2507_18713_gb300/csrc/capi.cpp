@@ -51,9 +51,9 @@ extern "C" salf_status salf_create(int32_t device, salf_ctx** out) {
   props.handleTypes = cudaMemHandleTypeNone;
   props.location.type = cudaMemLocationTypeDevice;
   props.location.id = device;
-  unsigned long long keep = kPoolKeep;
+  unsigned long long hold = kPoolHold;
   if ((e = cudaMemPoolCreate(&c->pool, &props)) != cudaSuccess ||
-      (e = cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+      (e = cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &hold)) != cudaSuccess) {
     salf_destroy(c);
     return salf_cuda_fail(e, "cudaMemPoolCreate");
   }

@@ -172,11 +172,13 @@ struct LaunchParams {
 
 // Device memory of scenes and of their builds comes from a pool of the
 // context's own (cudaMalloc and cudaFree took more than half of a 1M-voxel
-// rebuild).  What callers get pointers to, records and voxel order, comes from
-// cudaMalloc, as pool memory can be neither exported (cudaIpcGetMemHandle) nor
-// read by peers; freed blocks of it are kept for the next scene (a 162 MB block:
-// 40 us to allocate, 103 to free).  The context keeps this much of each.
-constexpr unsigned long long kPoolKeep = 512ull << 20, kBlocksKeep = 512ull << 20;
+// rebuild), which gives freed memory back while it holds more than kPoolHold,
+// memory in use included (a rebuild beside five other 1M-voxel scenes: 1210 us
+// with 512 MB, 859 with 1 GB).  What callers get pointers to, records and voxel
+// order, comes from cudaMalloc, as pool memory can be neither exported
+// (cudaIpcGetMemHandle) nor read by peers; up to kBlocksKeep bytes of freed blocks
+// are kept for the next scene (a 162 MB block: 40 us to allocate, 103 to free).
+constexpr unsigned long long kPoolHold = 1ull << 30, kBlocksKeep = 512ull << 20;
 
 struct DevBlock {
   void* p;

@@ -130,11 +130,17 @@ salf_status salf_scene_block(salf_scene* s, size_t bytes, void** p) {
 }
 
 // A scene's blocks go back to its context while the device is idle, the oldest
-// ones there to the device.
+// ones there to the device (and the scene's, where the list cannot grow).
 static void keep_blocks(salf_ctx* ctx, const std::vector<DevBlock>& blocks) {
   std::lock_guard<std::mutex> lk(ctx->blocks_mu);
-  size_t sum = 0;
+  try {
+    ctx->blocks.reserve(ctx->blocks.size() + blocks.size());
+  } catch (const std::bad_alloc&) {
+    for (const DevBlock& b : blocks) cudaFree(b.p);
+    return;
+  }
   ctx->blocks.insert(ctx->blocks.end(), blocks.begin(), blocks.end());
+  size_t sum = 0;
   for (const DevBlock& b : ctx->blocks) sum += b.bytes;
   while (sum > kBlocksKeep) {
     sum -= ctx->blocks.front().bytes;
